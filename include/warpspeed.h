@@ -177,7 +177,8 @@ typedef struct ws_profile {
   int64_t bitmap_bytes;      /* bitmap and page-flag bytes the plan's fields occupy        */
   int64_t passes;            /* scratch passes the plan needed                            */
   int64_t upload_bytes;      /* descriptor bytes the plan copied host -> device           */
-  int64_t row_reds;          /* 64-bit red.or issued by the row walk                      */
+  int64_t row_reds;          /* 64-bit red.or issued by the row walk (none where footprints
+                                are counted in closed form)                                */
   int64_t block_addresses;   /* (thread, access) address evaluations of the representative
                                 blocks (the exact per-address path)                        */
   float ms_create_host;      /* wall time of the plan's creation on the host: descriptor
@@ -185,7 +186,8 @@ typedef struct ws_profile {
   float ms_create_device;    /* wall time of the rest of the creation: device memory,
                                 descriptor upload, scratch zeroing, stream synchronisation */
   int64_t count_bytes;       /* bitmap bytes the counting kernel read: the pages the row walk
-                                flagged as written (every word for the other walks)        */
+                                flagged as written (every word for the other walks; none
+                                where footprints are counted in closed form)               */
 } ws_profile; /* 120 bytes */
 
 typedef struct ws_ctx ws_ctx;
@@ -273,9 +275,11 @@ typedef struct ws_plan_summary {
   int64_t fields;             /* field descriptors (a multi-dimensional candidate has two per field) */
   int64_t groups;             /* field groups */
   int64_t passes;             /* scratch passes */
-  int64_t enum_items, row_items, count_items;   /* work items of the three kernels */
+  /* work items of the three kernels: row_items are row-walk and closed-form items; count_items
+   * those of every bitmap, as the scratch accounts for them */
+  int64_t enum_items, row_items, count_items;
   int64_t access_entries;     /* folded access list entries after sharing */
-  int64_t interval_entries;   /* merged load run entries after sharing */
+  int64_t interval_entries;   /* merged load run and displacement entries after sharing */
   int64_t descriptor_bytes;   /* device bytes of descriptors, counters and results */
   int64_t scratch_bytes;      /* bitmap scratch the plan takes */
   int64_t bitmap_bytes;       /* bitmap bytes of all fields (what one pass would need) */

@@ -17,7 +17,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 CU_SOURCES = ["ws_kernels.cu", "ws_peaks.cu", "ws_noalloc.cu", "ws_validate.cu"]
 CPP_SOURCES = ["ws_plan.cpp", "ws_server.cpp"]
-HEADERS = ["ws_internal.h", "ws_kernels.h", "ws_host.h"]
+HEADERS = ["ws_internal.h", "ws_kernels.h", "ws_host.h", "ws_footprint.h"]
 
 
 def _newest_input() -> float:

@@ -140,7 +140,10 @@ struct ws_plan {
   ws::PinVec<ws::DGroup> hgrp;
   std::vector<char> grp_iv_ok;   // group allows the interval walk (used unless tune.walk asks otherwise)
   std::vector<char> grp_rows_ok; // group allows the row walk of levels 1-3
+  std::vector<char> grp_foot_ok; // levels the group may count in closed form (used with the row walk)
+  std::vector<int64_t> grp_foot_cost;    // closed form: estimated warp instructions per field
   std::vector<int64_t> grp_slots;        // row slots of the group's candidate
+  std::vector<int64_t> grp_blk_slots;    //   those of its representative block
   std::vector<ws::WarpClasses> grp_classes;  // block warp classes per group (used with the row walk)
   std::vector<int64_t> grp_winstr_rows;  // modelled (warp, instruction) pairs of levels 1-3
   // work-item sizes set by layout(): row slots per row-walk item (256, 512 or 1024),
@@ -158,7 +161,13 @@ struct ws_plan {
   std::vector<ws::DPass> passes;
   int64_t scratch_words = 0;
   size_t scratch_bytes = 0;
-  int64_t item_begin_end = 0, ritem_begin_end = 0, citem_begin_end = 0;
+  int64_t item_begin_end = 0, ritem_begin_end = 0, citem_begin_end = 0, fitem_begin_end = 0;
+  // counting items of every bitmap the plan accounts scratch for; citem_begin_end are those of
+  // the bitmaps it fills (levels counted in closed form fill none)
+  int64_t citems_accounted = 0;
+  int32_t foot_chunk = 1;        // closed-form items a warp takes at once
+  int32_t foot_stat = 1;         // items per group for what the closed-form walk does not count
+  int64_t own_budget = 0;        // owner-table entries the descriptor estimate allows for
   size_t grab_bytes = 0, counters_bytes = 0;
   // uploaded arrays that the plan owns until it is destroyed (their copies are asynchronous)
   ws::PinVec<ws::DCfg> up_cfg;
@@ -185,7 +194,7 @@ struct ws_plan {
   void layout();
   int upload_fields(cudaStream_t st);
   int grid_for(int threads, int64_t items, bool counting) const;
-  int grid_rows(int64_t items) const;
+  int grid_rows(int64_t items, int64_t fitems) const;
   int bank_shift() const;
   int enqueue(cudaStream_t st, std::vector<cudaEvent_t> *ev, ws_profile *prof);
   // Recorded after the descriptor uploads: launches on any stream wait for it (a graph

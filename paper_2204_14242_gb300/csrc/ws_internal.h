@@ -48,7 +48,7 @@ __host__ __device__ inline int64_t page_flag_words(int64_t words0, int64_t words
 // Montgomery 1994): with s = ceil(log2 d) and m = floor(2^32 (2^s - d) / d) + 1,
 // n / d = (umulhi(n, m) + n) >> s for every n < 2^31.
 struct FastDiv {
-  uint32_t d, m, s, pad;
+  uint32_t d, m, s;
 };
 
 // Thread groups of one candidate, flattened into one index space of "modelled warps":
@@ -82,6 +82,7 @@ struct DCfg {
   int32_t full_end;            // blocks in x that lie entirely inside N[0]
   FastDiv fd_rows, fd_b1;
   FastDiv fd_b2, fd_fold;      // for locating the row of a covering run
+  FastDiv fd_b1f, fd_b2f;      // grid rows and planes of one block (B[1], B[2] times the fold along that axis)
 };
 
 struct DField {
@@ -99,14 +100,23 @@ struct DField {
   int32_t n_load, n_store;// folded access counts (loads first, then stores)
   int32_t acc_begin;      // index into the DAcc array
   int32_t cfg;            // owning candidate
-  int32_t first_of_cfg;   // 1 if this is the candidate's first field (counts LUPs)
-  int32_t wide;           // a bitmap spans >= 2^32 bytes: 64-bit address path
-  int32_t lpa_log2p;      // log2 of P = lanes per thread-slice group for the load walk (P >= n_load, <= 32)
-  int32_t iv;             // interval walk possible: not wide and |elem_bytes * stride_x| <= 32
+  uint8_t first_of_cfg;   // 1 if this is the candidate's first field (counts LUPs)
+  uint8_t wide;           // a bitmap spans >= 2^32 bytes: 64-bit address path
+  uint8_t lpa_log2p;      // log2 of P = lanes per thread-slice group for the load walk (P >= n_load, <= 32)
+  uint8_t iv;             // interval walk possible: not wide and |elem_bytes * stride_x| <= 32
   int32_t iv_begin;       // first merged load interval (DIv array)
   int32_t n_iv;           // merged load intervals
-  int32_t rows_ok;        // stores: the row segments of one warp never share a sector
-  int32_t level_mask;     // levels served: 1 the representative block, 2 wave + y / z sets
+  uint8_t rows_ok;        // stores: the row segments of one warp never share a sector
+  uint8_t level_mask;     // levels served: 1 the representative block, 2 wave + y / z sets
+  uint8_t closed;         // closed-form footprints are exact: 1 wave + y / z sets, 2 the representative block
+  uint8_t zmove;          // closed form: the z set is the wave moved by whole planes, by zmove - 1 bytes modulo 128
+                          //   (0: it is not)
+  int32_t q;              // closed form: rows from plane to plane
+  uint32_t fq_m, fq_s;    //   and its FastDiv
+  int16_t n_dsp_l, n_dsp_s;   // closed form: displacements of the loads / of the stores (behind the intervals)
+  int32_t y_span_l, y_span_s; //   largest less smallest displacement within a plane (>= q: unknown)
+  uint8_t mult_l, mult_s;     //   fields of the group whose loads / stores this one's stand for (0: another one's do)
+  uint8_t pad8b[2];
   int32_t n_iv_unc;       // merged load intervals without a covering run (they come first)
   int32_t n_iv_zc;        // those covered from another z row (they come next; the rest last)
   int16_t cov_dy, cov_dz; // largest |row displacement| from an interval to its covering run
@@ -145,6 +155,15 @@ struct DIv {
 };
 constexpr int16_t kNoCover = -32768;
 
+// A displacement of the closed-form footprints: all raw loads (stores) of a field whose byte
+// offset is d rows plus a rest between clo and chi.  A field's displacements lie behind its
+// intervals in the DIv array, the loads' first.
+struct DDsp {
+  int32_t d, clo, chi;
+  int32_t pad;            // first entry: smallest clo; second: smallest displacement within a plane
+};
+static_assert(sizeof(DDsp) == sizeof(DIv), "displacements share the interval array");
+
 struct DHw {
   double clock_hz, l1_bytes, l2_bytes, bw_l2, bw_dram, fp_peak;
   double hit[4][3];
@@ -163,16 +182,20 @@ struct DGroup {
   int32_t f_begin;        // fields [f_begin, f_begin + f_count)
   int32_t f_count;
   int32_t acc_count;      // folded accesses of all its fields (<= kMaxFoldedAccesses)
-  int32_t first_of_cfg;   // the candidate's first group counts LUPs
-  int32_t uniform;        // all fields share element size and strides (and none is wide)
+  uint8_t first_of_cfg;   // the candidate's first group counts LUPs
+  uint8_t uniform;        // all fields share element size and strides (and none is wide)
+  uint8_t iv;             // uniform and every field allows the interval walk
+  uint8_t rows;           // levels 1-3 take the row walk (work items are chunks of row slots)
+  uint8_t levels;         // level mask of its fields (1 block, 2 wave + y / z, 3 both)
+  uint8_t first_wave;     // the candidate's first group with wave work counts the wave LUPs
+  uint8_t foot;           // closed-form footprints taken: 1 wave + y / z sets, 2 the representative block
+  uint8_t pad8;
+  int32_t f_parts;        // closed-form items per counted field (parts of its target rows)
+  uint32_t foot_fields;   // the fields counted (bit k: the group's k-th), the others being moved copies of them
   int32_t n_loads;        // folded loads of all its fields
   int32_t n_stores;       // folded stores of all its fields
-  int32_t iv;             // uniform and every field allows the interval walk
   int32_t n_iv;           // merged load intervals of all its fields
-  int32_t rows;           // levels 1-3 take the row walk (work items are chunks of row slots)
   int32_t n0_items;       // enumeration items of the representative block
-  int32_t levels;         // level mask of its fields (1 block, 2 wave + y / z, 3 both)
-  int32_t first_wave;     // the candidate's first group with wave work counts the wave LUPs
   // Representative-block warps to evaluate and the number of warps each one stands for
   // (warps with the same lane layout whose addresses differ by a multiple of the bank and
   // sector period give the same per-instruction counts); all warps, once each, unless the
@@ -180,7 +203,7 @@ struct DGroup {
   int32_t n_rep;
   uint8_t rep_warp[32];
   uint8_t rep_mult[32];
-  int32_t pad2;
+  int64_t fitem_begin;    // first closed-form item (field-major, f_parts per counted field)
 };
 
 // Classes of representative-block warps with identical per-instruction counts (host).
@@ -194,6 +217,7 @@ struct WarpClasses {
 struct DPass {
   int64_t item_lo, item_hi;    // enumeration items of the pass
   int64_t ritem_lo, ritem_hi;  // row-walk items of the pass
+  int64_t fitem_lo, fitem_hi;  // closed-form items of the pass
   int64_t citem_lo, citem_hi;  // counting items of the pass
   int32_t cf_lo, cf_hi;        // (candidate, field) index range
   int32_t grp_lo, grp_hi;      // field-group index range

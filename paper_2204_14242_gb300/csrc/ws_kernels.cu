@@ -6,9 +6,11 @@
 //                 the block bitmaps.  Wave / y / z sets of field groups that cannot take
 //                 the row walk: per modelled warp, as sector intervals of row segments
 //                 (segment walk) or address by address.
-//   rows_kernel   wave, y set and z set as whole grid rows: each merged load run of a
-//                 row is one sector range set with 64-bit red.or; per-warp store sectors
-//                 by floor sums (Sec. 4.4, closed-form counting instead of implicit sets).
+//   rows_kernel   wave, y set, z set and block footprints.  In closed form where a field's layout
+//                 allows it (ws_footprint.h; nearly always): counted row by row in registers,
+//                 without bitmaps.  Else as whole grid rows: each merged load run of a row is
+//                 one sector range set with 64-bit red.or; per-warp store sectors by floor
+//                 sums (Sec. 4.4, closed-form counting instead of implicit sets).
 //   count_kernel  popcounts of the bitmaps: unique sectors, unique 128 B lines (nibble
 //                 OR), y / z overlaps by AND / AND-NOT, reading only the pages the row
 //                 walk flagged, one warp per page.  Leaves the bitmaps and flags zeroed for
@@ -21,6 +23,7 @@
 
 #include <mutex>
 
+#include "ws_footprint.h"
 #include "ws_internal.h"
 #include "ws_kernels.h"
 
@@ -372,41 +375,12 @@ __device__ __forceinline__ bool segment_range(uint32_t th, uint32_t tt, int64_t 
   return true;
 }
 
-// Sum_{i=0}^{n-1} floor((a*i + b) / m) for a, b < m <= 32 and n < 2^31, by lattice-point
-// counting: with t = floor((a*(n-1) + b) / m) levels the sum equals t*n minus the
-// number of (i, k) with k <= t and a*i + b < k*m, which is the same kind of sum with the
-// roles of a and m exchanged; the exchanges follow Euclid's algorithm on (m, a), so all
-// divisors stay below 33.
-__device__ int64_t floor_sum_small(int64_t n, uint32_t m, uint32_t a, uint32_t b) {
-  int64_t res = 0, sgn = 1;
-  while (n > 0) {
-    if (a >= m) {
-      res += sgn * (int64_t)(a / m) * (n * (n - 1) / 2);
-      a %= m;
-    }
-    if (b >= m) {
-      res += sgn * (int64_t)(b / m) * n;
-      b %= m;
-    }
-    if (a == 0) break;
-    const int64_t t = ((int64_t)a * (n - 1) + b) / m;
-    if (t == 0) break;
-    res += sgn * t * n;
-    const uint32_t nb = m - b + a - 1;
-    n = t;
-    const uint32_t om = m;
-    m = a;
-    a = om;
-    b = nb;
-    sgn = -sgn;
-  }
-  return res;
-}
-
 // Sum_{i<n} floor((P*i + c) / 32) where every term's argument is >= 0 (P of any sign).
-// The multiple-of-32 part of P and c comes out in closed form; what is left is a sum
-// with a, b < 32 (none at all when P is a multiple of 32, as for every fp64 row of four
-// or more threads).
+// The multiple-of-32 part of P and c comes out in closed form.  What is left, a, b < 32, is
+// (a*i + b less its remainder) / 32 term by term; the remainders (a*i + b) mod 32 repeat after
+// 32 / g terms, g the lowest bit of a, running through all values that agree with b modulo g,
+// so only the terms of a last partial period (fewer than 8 for 4-byte elements, none at all
+// for fp64 rows of four or more threads) are added one by one.
 __device__ __forceinline__ int64_t sum_floor32(int64_t n, int64_t P, int64_t c) {
   if (n <= 0) return 0;
   if (P < 0) {
@@ -415,7 +389,13 @@ __device__ __forceinline__ int64_t sum_floor32(int64_t n, int64_t P, int64_t c) 
   }
   int64_t res = (P >> 5) * (n * (n - 1) / 2) + (c >> 5) * n;
   const uint32_t a = (uint32_t)(P & 31), b = (uint32_t)(c & 31);
-  if (a != 0) res += floor_sum_small(n, 32u, a, b);
+  if (a != 0) {
+    const uint32_t g = a & (0u - a), lp = 5u - (31u - __clz(g)), per = 1u << lp;
+    const uint32_t whole = per * (b & (g - 1u)) + g * (per * (per - 1u) / 2u);   // the remainders of one period
+    uint32_t part = 0, v = b;
+    for (uint32_t i = 0; i < ((uint32_t)n & (per - 1u)); ++i, v += a) part += v & 31u;
+    res += ((int64_t)a * (n * (n - 1) / 2) + (int64_t)b * n - (n >> lp) * (int64_t)whole - (int64_t)part) >> 5;
+  }
   return res;
 }
 
@@ -426,7 +406,7 @@ __device__ __forceinline__ int64_t sum_floor32(int64_t n, int64_t P, int64_t c) 
 // Segments repeat from block to block with the address step B0 * step, so each segment
 // position contributes two floor sums over the row's whole blocks; the block cut by N0
 // is counted directly.  A0 + step * x is the relative address of point x of the row.
-__device__ int64_t row_store_sectors(int64_t A0, int64_t step, int32_t B0, int32_t N0, int32_t full_end,
+__device__ __noinline__ int64_t row_store_sectors(int64_t A0, int64_t step, int32_t B0, int32_t N0, int32_t full_end,
                                      uint32_t t, uint32_t bxa, uint32_t bxb) {
   auto direct = [&](int64_t x0, int64_t x1) -> int64_t {
     const int64_t p = A0 + step * x0, q = A0 + step * x1;
@@ -1183,7 +1163,6 @@ __device__ __forceinline__ FastDiv make_fastdiv_dev(uint32_t d) {
   f.d = d;
   f.s = d <= 1u ? 0u : 32u - __clz(d - 1u);
   f.m = (uint32_t)((((unsigned long long)1 << 32) * (((unsigned long long)1 << f.s) - d)) / d + 1ull);
-  f.pad = 0u;
   return f;
 }
 
@@ -1231,7 +1210,715 @@ __device__ __forceinline__ bool row_interior(const DCfg &c, int lv, int32_t y, i
   return c.z_lo <= lo && hi <= up;
 }
 
-__global__ void __launch_bounds__(256, 4) rows_kernel(EnumArgs a) {
+
+// ---- closed-form footprints (ws_footprint.h) -------------------------------------------
+// A warp takes one part of one field's loads, stores and representative block.  It goes over a
+// task's target rows in units: the rows of a plane, repeated over the planes in which the
+// blocks' slabs let every state repeat (a block 64 planes deep has some 60 of them), whose
+// addresses differ by whole planes.  Parts share out the units in turn.  Inside a unit the warp
+// advances in windows of 32 rows, a lane per row.  First a lane per displacement looks up
+// which run of each level lands in the window and up to which row that stays so; displacements
+// constant over the window give their range to all rows with warp reductions, the others are
+// looked up row by row.  When everything is constant, the stretch up to the next change is
+// counted at once: its first 32 rows, then one period of the row addresses modulo a line (32
+// rows when the pitch is a multiple of four bytes) with the number of times each position
+// repeats.  Repeated planes likewise are counted once per position of the plane address modulo
+// a line; a window of few rows counts several of those positions at a time.
+constexpr int kFootRowCache = 64, kFootList = 48;
+
+// A task of a field: the loads or stores of the wave or of the block.
+struct FootTask {
+  const int4 *dsp;     // displacements
+  uint32_t base;       // address of x = 0 in row 0 (modulo 2^32; only its place in a line counts)
+  int32_t nd;          // their number (0: no such task)
+  int32_t P;           // pitch of a row
+  int32_t hmin;        // lowest byte of a row's ranges
+  int32_t pz, pzs;     // planes until their addresses repeat modulo a line (a power of two), log2
+  int32_t ymin;        // smallest displacement within a plane
+  int32_t rows;        // rows of a plane's unit that can hold anything
+  int32_t single;      // planes around a slab's end that units take one by one
+  int32_t zmove;       // wave loads: the z set's lines are the wave's, this many bytes on (-1: its own)
+  int32_t tr[4];       // target rows (foot_targets)
+};
+struct FootSmem {
+  FootGeo geo[2];      // wave, block: geometry of the warp's current field group
+  FootTask task[4];    // of its current field: wave loads, wave stores, block loads, block stores
+  // the row before a window: its ranges and levels (foot_join)
+  int32_t vl[3], vh[3];
+  uint32_t vm;
+  int ld;                                   // the unit's displacements
+  union {
+    unsigned long long sreq[kFootRowCache];   // store sectors of rows by what they depend on (foot_stats)
+    int4 list[kFootList];                     // the displacements left of a unit (foot_merge_list)
+  };
+};
+
+// Displacements up to which the rows of a short unit look them all up (a lane per row); with
+// more, and in long units, a lane per displacement first finds those that are constant over the
+// window.
+constexpr int kFootFew = 12;
+
+__device__ __forceinline__ void foot_sum(FootCounts &a, const FootCounts &b) {
+  a.sec += b.sec;
+  a.lin += b.lin;
+  a.ylin += b.ylin;
+  a.zlin += b.zlin;
+  a.ovy += b.ovy;
+  a.ovz += b.ovz;
+}
+
+// Counts a lane's target row t, `rows` times, where a level's first and last block rows leave a
+// gap between them (on this row or on another of the window): every displacement of the row and
+// of the row before it, piece by piece.  reps: the row's repeated planes (of at most `planes`).
+// Seldom taken and long: kept out of the walk's code, whose instructions have to stay in the SM's
+// caches.
+__device__ __noinline__ FootCounts foot_gaps(const FootGeo &g, const FootTask &k, const FootSmem &m, int nl, int32_t t,
+                                             uint32_t rows, int32_t reps, int32_t planes) {
+  FootCounts out = {0, 0, 0, 0, 0, 0};
+  if (reps <= 0 || rows == 0) return out;
+  const int nd = m.ld >= 0 ? m.ld : k.nd;
+  const int4 *const dsp = m.ld >= 0 ? m.list : k.dsp;
+  FootHull cur, prv;
+  cur.clear();
+  prv.clear();
+#pragma unroll 1
+  for (int e = 0; e < nd; ++e) {
+    const int4 v = dsp[e];
+    FootRow row;
+    foot_row(g, nl, t - v.x, false, row);
+    foot_add(row, nl, v.y, v.z, cur);
+    foot_row(g, nl, t - 1 - v.x, false, row);
+    foot_add(row, nl, v.y, v.z, prv);
+  }
+  const int32_t A = (int32_t)((k.base + (uint32_t)k.P * (uint32_t)t) & 127u), pzs = k.pzs;
+  const int32_t plane = (int32_t)(((uint32_t)k.P * (uint32_t)g.q) & 127u);
+  uint32_t zl = 0;
+#pragma unroll 1
+  for (int32_t i = 0; i < min(planes, k.pz); ++i) {
+    const uint32_t mult = rows * ((uint32_t)(reps - i + k.pz - 1) >> pzs);
+    if (mult) {
+      foot_count_pieces(cur, prv, A + i * plane, k.P, k.hmin, mult, out);
+      if (k.zmove > 0) {
+        FootCounts moved = {0, 0, 0, 0, 0, 0};
+        foot_count_pieces(cur, prv, A + i * plane + k.zmove, k.P, k.hmin, mult, moved);
+        zl += moved.lin;
+      }
+    }
+  }
+  if (k.zmove > 0) out.zlin = zl;
+  return out;
+}
+
+// Counts target rows [t_begin, t_end), each repeated over `reps` planes.  prime: the row before
+// t_begin may hold something (else it is empty in every plane).  Where the rows of whole planes
+// join (not every plane's stand alone), the first row's own predecessor lies before the repeated
+// planes and may differ from theirs: that row, t_first, is counted once, and the row q further
+// on, t_last, whose predecessor is the plane's last row, reps - 1 times in its place (kRowNone:
+// no such row among these).
+constexpr int32_t kRowNone = -kRowInf;
+__device__ __forceinline__ void foot_walk(const FootGeo &g, const FootTask &k, FootSmem &m, int nl, int32_t t_begin,
+                                          int32_t t_end, int32_t reps, bool prime, int32_t t_first, int32_t t_last,
+                                          FootCounts &out) {
+  const uint32_t lane = threadIdx.x & 31u;
+  __syncwarp();
+  if (lane == 0) {
+    m.vm = 0;
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      m.vl[l] = kHullLo;
+      m.vh[l] = kHullHi;
+    }
+  }
+  __syncwarp();
+  const int32_t t_lim = t_last != kRowNone ? t_last : t_end;   // (t_last is the last row)
+  const int32_t P = k.P, pzs = k.pzs, nres = min(reps, k.pz);
+  const int nd = m.ld >= 0 ? m.ld : k.nd;
+  const int4 *const dsp = m.ld >= 0 ? m.list : k.dsp;
+  const int32_t plane = (int32_t)(((uint32_t)P * (uint32_t)g.q) & 127u);
+  // the row before the first one is looked up too, but not counted
+  int32_t t = t_begin - (prime ? 1 : 0);
+#pragma unroll 1
+  for (;;) {
+  int gap = 0;   // rows of a window that takes foot_gaps (called outside the windows' loop)
+#pragma unroll 1
+  while (t < t_end) {
+    FootHull U;
+    U.clear();
+    const int32_t left = t_end - t;
+    bool varies = true;
+    int32_t nb = kRowInf;   // first row at which a displacement constant over the window changes
+    uint32_t todo = (1u << min(nd, kFootFew)) - 1u;   // displacements left to the rows (lane j: of the j-th 32)
+    if (left > 32 || nd > kFootFew) {
+      uint32_t some = 0;
+#pragma unroll 1
+      for (int e0 = 0; e0 < nd; e0 += 32) {
+        bool part = false;
+        if (e0 + (int)lane < nd) {
+          const int4 v = dsp[e0 + (int)lane];
+          FootRow row;
+          const int32_t nx = foot_row(g, nl, t - v.x, true, row);
+          const int32_t nt = nx == kRowInf ? kRowInf : nx + v.x;
+          part = nt < t + min(32, left);
+          if (!part) {
+            nb = min(nb, nt);
+            foot_add(row, nl, v.y, v.z, U);
+          }
+        }
+        const uint32_t pm = __ballot_sync(FULL, part);
+        if (lane == (uint32_t)e0 >> 5) todo = pm;
+        some |= pm;
+      }
+      varies = some != 0u;
+      // the constant displacements' ranges, for all rows
+      nb = __reduce_min_sync(FULL, nb);
+#pragma unroll
+      for (int l = 0; l < 3; ++l) {
+        if (l > 0 && nl == 1) break;
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+          if (__any_sync(FULL, U.lo[l][c] <= U.hi[l][c])) {
+            U.lo[l][c] = __reduce_min_sync(FULL, U.lo[l][c]);
+            U.hi[l][c] = __reduce_max_sync(FULL, U.hi[l][c]);
+          }
+      }
+    }
+    if (varies) {
+#pragma unroll 1
+      for (int e0 = 0; e0 < nd; e0 += 32) {
+        uint32_t pm = __shfl_sync(FULL, todo, e0 >> 5);
+#pragma unroll 1
+        while (pm) {
+          const int4 v = dsp[e0 + __ffs(pm) - 1];
+          pm &= pm - 1;
+          FootRow row;
+          foot_row(g, nl, t + (int32_t)lane - v.x, false, row);
+          foot_add(row, nl, v.y, v.z, U);
+        }
+      }
+    }
+    int32_t cl[3], ch[3], pl[3], ph[3];
+    const uint32_t um = foot_join(U, nl, cl, ch);
+    uint32_t um1 = __shfl_up_sync(FULL, um, 1);
+    if (lane == 0) um1 = m.vm;
+    const int32_t tl = t + (int32_t)lane;
+    const bool act = (um | um1) != 0u && (int32_t)lane < left && tl >= t_begin;
+    uint32_t levels = __reduce_or_sync(FULL, act ? um | um1 : 0u);
+    int32_t n = min(32, left), rest = 0;
+    if (!varies) {
+      // constant up to row nb (row t_last, if among them, is left to the next window)
+      n = max(n, min(nb, t_lim) - t);
+      rest = n - 32;
+    }
+    if (levels & 8u) {
+      gap = n;
+    } else if (levels) {
+      int32_t rl = !act ? 0 : tl == t_last ? reps - 1 : tl == t_first ? 1 : reps;
+      {
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+          pl[l] = __shfl_up_sync(FULL, cl[l], 1);
+          ph[l] = __shfl_up_sync(FULL, ch[l], 1);
+          if (lane == 0) {
+            pl[l] = m.vl[l];
+            ph[l] = m.vh[l];
+          }
+        }
+        int32_t A = (int32_t)((k.base + (uint32_t)P * (uint32_t)tl) & 127u);
+        const uint32_t am = __ballot_sync(FULL, act);
+        const int first = __ffs(am) - 1, span = 32 - __clz(am) - first;
+        __syncwarp();
+        if ((int)lane == min(n, 32) - 1) {
+#pragma unroll
+          for (int l = 0; l < 3; ++l) {
+            m.vl[l] = cl[l];
+            m.vh[l] = ch[l];
+          }
+        }
+        __syncwarp();
+        int32_t i0 = 0, di = 1;
+        if (nres > 1 && span <= 16) {
+          // few rows: 32 / w plane positions at a time, w >= the rows
+          const int ws = span <= 1 ? 0 : 32 - __clz(span - 1), j = (int)lane & ((1 << ws) - 1);
+#pragma unroll
+          for (int l = 0; l < 3; ++l) {
+            if (l > 0 && nl == 1) break;
+            cl[l] = __shfl_sync(FULL, cl[l], first + j);
+            ch[l] = __shfl_sync(FULL, ch[l], first + j);
+            pl[l] = __shfl_sync(FULL, pl[l], first + j);
+            ph[l] = __shfl_sync(FULL, ph[l], first + j);
+          }
+          A = __shfl_sync(FULL, A, first + j);
+          rl = __shfl_sync(FULL, rl, first + j);
+          if (j >= span) rl = 0;
+          i0 = (int32_t)lane >> ws;
+          di = 32 >> ws;
+        }
+        if (k.zmove < 0) levels |= 16u;
+        // the window's rows, then one period of the positions of the rows behind it
+        uint32_t times = 1;
+        const int32_t pers = 5 + (P & 1 ? 2 : P & 2 ? 1 : 0), per = 1 << pers;
+        int32_t j0 = -32;
+#pragma unroll 1
+        for (;;) {
+          if (rl > 0)
+#pragma unroll 1
+            for (int32_t i = i0; i < nres; i += di) {
+              const uint32_t mult = times * ((uint32_t)(rl - i + k.pz - 1) >> pzs);
+              if (mult) {
+                foot_count(cl, ch, pl, ph, A + i * plane, P, k.hmin, mult, levels, out);
+                if (k.zmove > 0 && (levels & 1u))
+                  out.zlin += mult * foot_count_lines(cl[0], ch[0], pl[0], ph[0], A + i * plane + k.zmove, P, k.hmin);
+              }
+            }
+          j0 += 32;
+          if (j0 >= min(per, rest)) break;
+          const int32_t j = j0 + (int32_t)lane;
+          times = j < rest ? (uint32_t)(rest - j + per - 1) >> pers : 0u;
+          rl = reps;
+          A = (int32_t)((k.base + (uint32_t)P * (uint32_t)(t + 32 + j)) & 127u);
+          i0 = 0;
+          di = 1;
+#pragma unroll
+          for (int l = 0; l < 3; ++l) {
+            cl[l] = pl[l] = m.vl[l];   // the state of the window's last row
+            ch[l] = ph[l] = m.vh[l];
+          }
+        }
+      }
+    }
+    // the state of the stretch's last row (a constant stretch: of any of its rows)
+    __syncwarp();
+    if ((int)lane == min(n, 32) - 1) {
+      m.vm = um;
+      if (!levels || (levels & 8u)) {
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+          m.vl[l] = cl[l];
+          m.vh[l] = ch[l];
+        }
+      }
+    }
+    __syncwarp();
+    if (gap) break;
+    t += n;
+  }
+  if (!gap) break;
+  // the window's rows, then one period of the positions of the rows behind it
+  {
+    const int32_t tl = t + (int32_t)lane;
+    const int32_t rl = (int32_t)lane >= gap || tl < t_begin ? 0
+                       : tl == t_last                       ? reps - 1
+                       : tl == t_first                      ? 1
+                                                            : reps;
+    foot_sum(out, foot_gaps(g, k, m, nl, tl, 1u, rl, reps));
+    const int32_t pers = 5 + (P & 1 ? 2 : P & 2 ? 1 : 0), rest = gap - 32;
+#pragma unroll 1
+    for (int32_t j = (int32_t)lane; j < min(1 << pers, rest); j += 32)
+      foot_sum(out, foot_gaps(g, k, m, nl, t + 32 + j, (uint32_t)(rest - j + (1 << pers) - 1) >> pers, reps, reps));
+  }
+  t += gap;
+  }
+}
+
+// floor(a / q) and the remainder of any a > -2^30
+__device__ __forceinline__ int32_t foot_rem(int32_t a, const FootGeo &g) {
+  const int32_t z = a >= 0 ? (int32_t)foot_div((uint32_t)a, g.fq_m, g.fq_s)
+                           : -(int32_t)foot_div((uint32_t)(g.q - 1 - a), g.fq_m, g.fq_s);
+  return a - z * g.q;
+}
+
+// The displacements of a unit of n rows from t - 1 on: those whose source rows hold nothing are
+// left out, those that look up the same states throughout (equal row in a plane of the same
+// slab, as the out-of-plane arms of a star on deep blocks) become one with their common range of
+// rests.  m.ld = -1: too many, the task's own list stands.
+__device__ __forceinline__ void foot_merge_list(const FootGeo &g, const FootTask &k, FootSmem &m, int32_t t, int32_t n) {
+  const uint32_t lane = threadIdx.x & 31u;
+  int have = 0;
+  __syncwarp();
+#pragma unroll 1
+  for (int e0 = 0; e0 < k.nd && have >= 0; e0 += 32) {
+    const int e = e0 + (int)lane;
+    int4 v = make_int4(0, 0, 0, 0);
+    int32_t key[4] = {-1 - (int32_t)lane, -2, -2, -2};
+    bool on = false;
+    if (e < k.nd) {
+      v = __ldg(k.dsp + e);
+      on = foot_key(g, t - 1 - v.x, n, key);
+    }
+    uint32_t same = __match_any_sync(FULL, key[0]);
+    if (__any_sync(FULL, on && (same & (same - 1u)))) {
+      same &= __match_any_sync(FULL, key[1]) & __match_any_sync(FULL, key[2]) & __match_any_sync(FULL, key[3]);
+      v.y = __reduce_min_sync(same, v.y);
+      v.z = __reduce_max_sync(same, v.z);
+    }
+    const bool keep = on && (int)lane == __ffs(same) - 1;
+    const uint32_t km = __ballot_sync(FULL, keep);
+    const int at = have + __popc(km & ((1u << lane) - 1u));
+    have += __popc(km);
+    if (have > kFootList) have = -1;
+    else if (keep) m.list[at] = v;
+  }
+  if (lane == 0) m.ld = have;
+  __syncwarp();
+}
+
+// One task's share: planes in units, the ones around a slab's ends one by one and the others
+// between them together; the parts take equal numbers of units in order.
+__device__ __noinline__ FootCounts foot_task(FootSmem &m, int kind, int part, int parts) {
+  const uint32_t lane = threadIdx.x & 31u;
+  FootCounts out = {0, 0, 0, 0, 0, 0};
+  const FootGeo &g = m.geo[kind >> 1];
+  const FootTask &k = m.task[kind];
+  const int nl = kind == 0 ? 3 : 1;
+  // with an empty row to spare on both sides of its rows every plane's stand alone
+  const int32_t rows = k.rows, q = g.q;
+  const bool isolated = rows + 1 <= q;
+#pragma unroll 1
+  for (int s = 0; s < 4; s += 2) {
+    const int32_t t0 = k.tr[s], t1 = k.tr[s + 1];
+    if (t0 >= t1) continue;
+    // planes begin where the first displaced plane begins, so that a plane's rows with points
+    // are not cut in two
+    const int32_t ph0 = foot_rem(t0 - k.ymin, g), np = (int32_t)foot_div((uint32_t)(t1 - t0 + ph0 + q - 1), g.fq_m, g.fq_s);
+    int32_t a = 0, b = np;
+    uint32_t cut = 1, piece = 0;
+    if (parts > 1) {
+      // planes before unit u: `single` units of one plane and one of the rest per slab, and
+      // `single` at the end (any rising cut of the planes is correct); where the wave's loads have
+      // more parts than units the units' rows are cut, too
+      const uint32_t n = (uint32_t)np, one = min((uint32_t)k.single, n), n1 = n - one;
+      const uint32_t per = (uint32_t)k.single + 1u, b2f = (uint32_t)g.b2f;
+      const bool deep = b2f > per;
+      const uint32_t full = deep ? foot_div(n1, g.fb2_m, g.fb2_s) : 0u;
+      const uint32_t u1 = deep ? full * per + min(n1 - full * b2f, per) : n1, units = u1 + one;
+      cut = kind == 0 ? max(1u, (uint32_t)parts / units) : 1u;
+      const uint32_t pp = min((uint32_t)parts / cut, units), pu = (uint32_t)part / cut;
+      piece = (uint32_t)part - pu * cut;
+      if (pu >= pp) continue;
+      // (units and pieces stay below 2^25, parts below 2^7)
+#pragma unroll 1
+      for (uint32_t i = 0; i < 2u; ++i) {
+        const uint32_t u = units * (pu + i) / pp, sl = deep ? u / per : 0u;
+        const int32_t pl = (int32_t)(u >= u1 ? n1 + (u - u1) : min(n1, deep ? sl * b2f + (u - sl * per) : u));
+        if (i == 0u) a = pl;
+        else b = pu + 1u == pp ? np : pl;
+      }
+    }
+    int32_t t = max(t0, t0 - ph0 + a * q), ph = a == 0 ? ph0 : 0;
+    const int32_t te = min(t1, t0 - ph0 + b * q);
+#pragma unroll 1
+    while (t < te) {
+      if (isolated && ph >= rows) {   // the rest of the plane is empty
+        t += q - ph;
+        ph = 0;
+        continue;
+      }
+      int32_t n = 1, end = min(te, t + (q - ph));
+      if (ph == 0 && te - t >= 2 * q) {
+        int32_t r = kRowInf;
+#pragma unroll 1
+        for (int e = (int)lane; e < k.nd; e += 32) r = min(r, foot_repeat(g, t - __ldg(&k.dsp[e].x)));
+        r = __reduce_min_sync(FULL, r);
+        n = min(r, (int32_t)foot_div((uint32_t)(te - t), g.fq_m, g.fq_s));
+        end = t + n * q;
+      }
+      int32_t from = t, stop = isolated ? min(end, t + (rows - ph)) : n > 1 ? t + q : end;
+      const bool wrap = n > 1 && !isolated;
+      bool prime = !(isolated && ph == 0);
+      if (cut > 1u) {
+        const uint32_t len = (uint32_t)(stop - t);
+        from = t + (int32_t)(len * piece / cut);
+        stop = t + (int32_t)(len * (piece + 1u) / cut);
+        prime = prime || from > t;
+      }
+      if (from < stop) {
+        const int32_t first = wrap && from == t ? t : kRowNone, last = wrap && stop == t + q ? stop : kRowNone;
+        if (last != kRowNone) stop = last + 1;
+        foot_merge_list(g, k, m, from, stop - from + 1);
+        if (m.ld != 0) foot_walk(g, k, m, nl, from, stop, n, prime, first, last, out);
+      }
+      ph = 0;
+      t = end;
+    }
+  }
+  return out;
+}
+
+// Counters of a task's sectors and lines (wave loads, wave stores, block loads, block stores), and
+// of the wave's loads' y and z lines and overlaps.
+__constant__ uint32_t kFootDst[4] = {C_W_LS | C_W_LL << 8, C_W_SS | C_W_SL << 8, C_BLK_LS | C_BLK_LL << 8,
+                                     C_BLK_SS | C_BLK_SL << 8};
+constexpr uint32_t kFootDst3 = C_Y_LINES | C_Z_LINES << 8 | C_OV_Y << 16 | (uint32_t)C_OV_Z << 24;
+
+// What the walk does not count of a field group, once per group: the wave's lattice updates, the
+// valid address evaluations (threads of each level with all folded points valid and with fewer,
+// at the domain's end) and the per-warp store sectors of the wave (the partial-store request
+// volume).  The latter take a lane per thread row, in closed form.  A row's count depends on
+// the store's address only modulo 32 bytes and on the first valid folded point it needs, so the
+// group's stores that agree on both are counted together; and on the row only through its start
+// modulo 32 bytes, t * B0 modulo 32 and the block run (whole, or cut at the wave's first or last
+// block), so the warp keeps the counts it has by those.
+__device__ __noinline__ void foot_stats(const EnumArgs &a, const DGroup &G, unsigned long long *cache, int part, int parts) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const DCfg &c = a.cfg[G.cfg];
+  unsigned long long *const cnt = (unsigned long long *)(a.counters + (int64_t)G.cfg * N_COUNTERS);
+  if (part == 0) {
+    const int32_t rest = c.fold_axis ? c.N[c.fold_axis] % c.fold : 0;
+    // a lane per term, then a lane per (level, all or only partly valid threads)
+    __syncwarp();
+    if (lane < 24u) cache[lane] = (unsigned long long)foot_thread_term(c, (int)(lane % 12u), lane >= 12u);
+    __syncwarp();
+    unsigned long long th = 0;
+    if (lane < 6u) {
+      const uint32_t l = lane >> 1;
+      for (uint32_t j = l == 0 ? 0u : l == 1 ? 2u : 6u; j < (l == 0 ? 2u : l == 1 ? 6u : 12u); ++j)
+        th += cache[j + ((lane & 1u) ? 12u : 0u)];
+    }
+    __syncwarp();
+    int32_t lf = 0, lp = 0, sf = 0, sp = 0;
+    if ((int)lane < G.f_count) {
+      const DField &f = a.fld[G.f_begin + (int)lane];
+      lf = f.cnt_load[c.fold];
+      sf = f.cnt_store[c.fold];
+      lp = f.cnt_load[rest];
+      sp = f.cnt_store[rest];
+    }
+    lf = __reduce_add_sync(FULL, lf);
+    lp = __reduce_add_sync(FULL, lp);
+    sf = __reduce_add_sync(FULL, sf);
+    sp = __reduce_add_sync(FULL, sp);
+    unsigned long long ad = 0, lups = 0;
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      const unsigned long long all = __shfl_sync(FULL, th, 2 * l), few = __shfl_sync(FULL, th, 2 * l + 1);
+      ad += (all - few) * (unsigned long long)(lf + (l == 0 ? sf : 0)) +
+            few * (unsigned long long)(lp + (l == 0 ? sp : 0));
+      if (l == 0) lups = (all - few) * (unsigned long long)c.fold + few * (unsigned long long)rest;
+    }
+    if (lane == 0) {
+      if (ad) atomicAdd(cnt + C_ADDR, ad);
+      if (G.first_wave && lups) atomicAdd(cnt + C_LUPS_WAVE, lups);
+    }
+  }
+  unsigned long long sum = 0;
+  const DField &F0 = a.fld[G.f_begin];
+  const int64_t es = F0.esize, sxe = es * F0.stride[0];
+  const int32_t slots = (int32_t)c.rows_slot_end[0];
+  const uint32_t gx = (uint32_t)c.g[0], gy = (uint32_t)c.g[1];
+  const uint32_t py = (uint32_t)(es * F0.stride[1]) & 31u, pz = (uint32_t)(es * F0.stride[2]) & 31u;
+  const uint32_t w0 = (uint32_t)c.s, w1 = (uint32_t)(c.s + c.weff);
+  __syncwarp();
+  for (int i = (int)lane; i < kFootRowCache; i += 32) cache[i] = ~0ull;
+  __syncwarp();
+  // the group's distinct (address modulo 32, first needed point) codes, a lane each, and how many
+  // stores have them; taken through the rows when 32 might not hold more, and at the end
+  uint32_t code = 0, times = 0;
+  int nu = 0, k = 0, j0 = 0;   // codes held; next field and its next store
+#pragma unroll 1
+  for (;;) {
+    // up to 32 stores: of one field, or of several in a row
+    uint32_t mine = 0xffffffffu;
+    int have = 0;
+#pragma unroll 1
+    while (k < G.f_count && have < 32) {
+      const DField &F = a.fld[G.f_begin + k];
+      const int take = min(32 - have, F.n_store - j0), at = (int)lane - have;
+      if (at >= 0 && at < take) {
+        const DAcc x = a.acc[F.acc_begin + F.n_load + j0 + at];
+        mine = (uint32_t)((x.boff + F.base) & 31) | ((uint32_t)x.kmin << 5);
+      }
+      have += take;
+      j0 += take;
+      if (j0 >= F.n_store) {
+        ++k;
+        j0 = 0;
+      }
+    }
+    const uint32_t same = __match_any_sync(FULL, mine);
+    uint32_t todo = __ballot_sync(FULL, (int)lane < have && (int)lane == __ffs(same) - 1);
+    if (have == 0 || nu + __popc(todo) > 32) {
+      const int64_t n0 = ((int64_t)slots + 31) / 32;   // this part's rows, 32 at a time
+      for (int32_t r = (int32_t)(n0 * part / parts); r < (int32_t)(n0 * (part + 1) / parts) && nu > 0; ++r) {
+        const int32_t slot = 32 * r + (int32_t)lane;
+        const uint32_t pq = fdiv((uint32_t)slot, c.fd_rows);
+        const uint32_t t = (uint32_t)slot - pq * (uint32_t)c.rows_per_blk;
+        const uint32_t R = (uint32_t)c.rows_R_lo[0] + pq;
+        const uint32_t bz = fdiv(R, c.fd_gy), by = R - bz * gy, rb0 = R * gx;
+        const uint32_t bxa = w0 > rb0 ? w0 - rb0 : 0u, bxb = min(w1 - rb0, gx);   // (a row of the wave: not empty)
+        const uint32_t tz = fdiv(t, c.fd_b1), ty = t - tz * (uint32_t)c.B[1];
+        int32_t y = (int32_t)(by * (uint32_t)c.B[1] + ty), z = (int32_t)(bz * (uint32_t)c.B[2] + tz);
+        if (c.fold_axis == 1) y *= c.fold;
+        if (c.fold_axis == 2) z *= c.fold;
+        int kv = c.fold_axis == 1   ? min(c.fold, c.N[1] - y)
+                 : c.fold_axis == 2 ? min(c.fold, c.N[2] - z)
+                                    : 1;
+        if (slot >= slots || y >= c.N[1] || z >= c.N[2]) kv = 0;
+        const uint32_t a0 = py * (uint32_t)y + pz * (uint32_t)z;
+        // one block run starts inside a block row, one ends inside one
+        const uint32_t tag0 = (((t * (uint32_t)c.B[0]) & 31u) << 5) | (bxa > 0u ? 1u << 10 : 0u) | (bxb < gx ? 1u << 11 : 0u);
+#pragma unroll 1
+        for (int u = 0; u < nu; ++u) {
+          const uint32_t cd = __shfl_sync(FULL, code, u), ct = __shfl_sync(FULL, times, u);
+          if ((int32_t)(cd >> 5) >= kv) continue;
+          const uint32_t A0 = (a0 + cd) & 31u, tag = tag0 | A0, at = (tag * 0x9E3779B1u) >> 26;
+          const unsigned long long hit = cache[at];
+          uint32_t val = (uint32_t)hit;
+          if ((uint32_t)(hit >> 32) != tag) {
+            val = (uint32_t)row_store_sectors((int64_t)A0, sxe, c.B[0], c.N[0], c.full_end, t, bxa, bxb);
+            cache[at] = ((unsigned long long)tag << 32) | val;
+          }
+          sum += (unsigned long long)val * ct;
+        }
+        __syncwarp();
+      }
+      nu = 0;
+      if (have == 0) break;
+    }
+#pragma unroll 1
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const uint32_t cd = __shfl_sync(FULL, mine, src), n = (uint32_t)__popc(__shfl_sync(FULL, same, src));
+      const bool held = (int)lane < nu && code == cd;
+      if (__any_sync(FULL, held)) {
+        if (held) times += n;
+      } else {
+        if ((int)lane == nu) {
+          code = cd;
+          times = n;
+        }
+        ++nu;
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(FULL, sum, o);
+  if (lane == 0 && sum) atomicAdd(cnt + C_W_SREQ, sum);
+}
+
+// Geometry of a field group: the wave and its y and z sets, and the representative block.
+__device__ __noinline__ void foot_setup(FootSmem &m, const DCfg &c, const DField &F) {
+  const uint32_t lane = threadIdx.x & 31u;
+  __syncwarp();
+  const int32_t esx = (int32_t)(F.esize * F.stride[0]);
+  if (lane < 6) foot_level(m.geo[lane < 3 ? 0 : 1], c, F.q, esx, lane >= 3, (int)(lane < 3 ? lane : lane - 3));
+  __syncwarp();
+  if (lane < 2) {
+    FootGeo &g = m.geo[lane];
+    foot_finish(g, c, F.q, esx);
+    g.fq_m = F.fq_m;
+    g.fq_s = F.fq_s;
+  }
+  __syncwarp();
+}
+
+// The tasks of a field, a lane each.
+__device__ __noinline__ void foot_field(const EnumArgs &a, FootSmem &m, const DField &F, uint32_t foot) {
+  const uint32_t lane = threadIdx.x & 31u;
+  __syncwarp();
+  if (lane < 4) {
+    FootTask &k = m.task[lane];
+    const bool st = lane & 1u, blk = lane >= 2u;
+    const FootGeo &g = m.geo[lane >> 1];
+    const int nd = st ? F.n_dsp_s : F.n_dsp_l;
+    const int32_t P = (int32_t)(F.esize * F.stride[1]);
+    k.nd = (foot & (blk ? 2u : 1u)) && (st ? F.mult_s : F.mult_l) ? nd : 0;
+    if (k.nd > 0) {
+      // the list is sorted by d; its first entry also holds the smallest clo, its second the
+      // smallest displacement within a plane
+      const int4 *const dsp = reinterpret_cast<const int4 *>(a.iv + F.iv_begin + F.n_iv + (st ? F.n_dsp_l : 0));
+      const int4 d0 = __ldg(dsp), d1 = __ldg(dsp + (nd > 1 ? 1 : 0));
+      const uint32_t pb = ((uint32_t)P * (uint32_t)g.q) & 127u;
+      k.dsp = dsp;
+      k.base = (uint32_t)(F.base + (int64_t)F.esize * (F.stride[1] * g.y0 + F.stride[2] * g.z0));
+      k.P = P;
+      k.hmin = d0.w;
+      k.pzs = pb ? 8 - __ffs(pb) : 0;
+      k.pz = 1 << k.pzs;
+      k.ymin = nd > 1 ? d1.w : d0.x;
+      // the displaced rows with points and the cell behind them
+      k.rows = g.y_act + (st ? F.y_span_s : F.y_span_l) + 1;
+      k.single = (int32_t)foot_div((uint32_t)(__ldg(&dsp[nd - 1].x) - d0.x), g.fq_m, g.fq_s) + 1;
+      k.zmove = lane == 0 ? (int32_t)F.zmove - 1 : -1;
+      foot_targets(g, lane == 0 ? 3 : 1, d0.x, __ldg(&dsp[nd - 1].x), k.zmove < 0, k.tr);
+    }
+  }
+  __syncwarp();
+}
+
+// The closed-form items of a pass: warps take fchunk consecutive ones at a time and keep the
+// geometry of a field group while they stay in it; before them fstat items per group for
+// what the walk does not count.
+__device__ __forceinline__ void foot_items(const EnumArgs &a, FootSmem &m) {
+  const uint32_t lane = threadIdx.x & 31u;
+  int cur = -1;
+#pragma unroll 1
+  for (;;) {
+    unsigned long long i0 = 0;
+    if (lane == 0) i0 = atomicAdd(a.fgrab, (unsigned long long)a.fchunk);
+    const int64_t it0 = a.fitem_lo + (int64_t)__shfl_sync(FULL, i0, 0);
+    const int64_t ns = (int64_t)(a.grp_hi - a.grp_lo) * a.fstat;
+    const int64_t it_end = a.fitem_hi + ns;
+    if (it0 >= it_end || a.fitem_hi == a.fitem_lo) break;
+    const int64_t it1 = min(it0 + a.fchunk, it_end);
+#pragma unroll 1
+    for (int64_t it = it0; it < it1; ++it) {
+      if (it < a.fitem_lo + ns) {
+        const int i = (int)(it - a.fitem_lo), gi = i / a.fstat;
+        const DGroup &G = a.grp[a.grp_lo + gi];
+        if (G.foot & 1) foot_stats(a, G, m.sreq, i - gi * a.fstat, a.fstat);
+        continue;
+      }
+      const int64_t itf = it - ns;
+      const int gi = a.own_foot[itf];
+      const DGroup &G = a.grp[gi];
+      const int parts = G.f_parts, o = (int)(itf - G.fitem_begin), nth = o / parts, p = o - nth * parts;
+      // the nth counted field of the group
+      const uint32_t ff = G.foot_fields;
+      const int k = __ffs(__ballot_sync(FULL, ((ff >> lane) & 1u) && __popc(ff & ((1u << lane) - 1u)) == nth)) - 1;
+      const DField &F = a.fld[G.f_begin + k];
+      if (gi != cur) {
+        cur = gi;
+        foot_setup(m, a.cfg[G.cfg], F);
+      }
+      foot_field(a, m, F, G.foot);
+      const bool zs = F.zmove == 1;   // the z set's lines are the wave's
+      unsigned long long *const cnt = (unsigned long long *)(a.counters + (int64_t)G.cfg * N_COUNTERS);
+      // a task's units are shared out among the parts
+#pragma unroll 1
+      for (int i = 0; i < 4; ++i) {
+        int kind = i;   // not a constant: the walk's code, made once, has to stay in the instruction cache
+        asm volatile("" : "+r"(kind));
+        const bool st = kind & 1;
+        if (m.task[kind].nd == 0) continue;
+        // (the kinds' first parts, often the longest, fall to different warps)
+        const int at = kind == 0 ? p : kind == 1 ? parts - 1 - p : p >= parts / 2 ? p - parts / 2 : p + parts - parts / 2;
+        const FootCounts n = foot_task(m, kind, at, parts);
+        // lane i adds the i-th count; the counters of each kind, a byte each
+        const uint32_t v0 = __reduce_add_sync(FULL, n.sec), v1 = __reduce_add_sync(FULL, n.lin);
+        uint32_t v = lane == 0 ? v0 : v1, dst = lane < 2 ? (kFootDst[kind] >> (8 * lane)) & 255u : 255u;
+        if (kind == 0) {
+          const uint32_t v2 = __reduce_add_sync(FULL, n.ylin), v3 = zs ? v1 : __reduce_add_sync(FULL, n.zlin);
+          const uint32_t v4 = __reduce_add_sync(FULL, n.ovy), v5 = __reduce_add_sync(FULL, n.ovz);
+          v = lane < 2 ? v : lane == 2 ? v2 : lane == 3 ? v3 : lane == 4 ? v4 : v5;
+          if (lane >= 2 && lane < 6) dst = (uint32_t)(kFootDst3 >> (8 * (lane - 2))) & 255u;
+        }
+        if (dst != 255u && v) atomicAdd(cnt + dst, (unsigned long long)v * (st ? F.mult_s : F.mult_l));
+      }
+    }
+  }
+}
+
+// Row items first (CTAs), then the closed-form items (warps).  Bound by instruction fetch and the
+// latency of a warp's own chain: a unit runs a few thousand instructions once, so the code has to
+// stay in the SM's instruction cache (one copy of the walk, rare paths out of line), and two
+// CTAs an SM with 128 registers beat three or four that spill (0.23 against 0.29 and 0.35 ms,
+// 25-point sweep of 755).  Footprints of 755 25-point candidates at 640 x 512 x 512: 0.193 ms of
+// red.or and 0.092 ms of counting 179 MB of bitmaps -> 0.230 and 0.018 ms; 755 lattice Boltzmann
+// candidates: 1.163 and 0.984 -> 0.252 and 0.002 ms (3.66 GB of bitmaps not read, fields that are
+// whole-line copies counted once); 4,000 mixed candidates: 2.66 and 1.32 -> 1.90 and 0.06 ms.
+__global__ void __launch_bounds__(256, 2) rows_kernel(EnumArgs a) {
+
   __shared__ DCfg s_c;
   __shared__ DGroup s_g;
   __shared__ DField s_fk[kMaxGroupFields];
@@ -1241,7 +1928,7 @@ __global__ void __launch_bounds__(256, 4) rows_kernel(EnumArgs a) {
   __shared__ int32_t s_idst[3][kMaxGroupFields];
   __shared__ int32_t s_cov[5];
   __shared__ uint8_t s_af[kMaxFoldedAccesses];
-  __shared__ int64_t s_boff[kMaxFoldedAccesses];
+  __shared__ __align__(16) int64_t s_boff[kMaxFoldedAccesses];
   __shared__ uint8_t s_kmin[kMaxFoldedAccesses];
   __shared__ int32_t s_gad[2][17];
   __shared__ int32_t s_gwi[2];
@@ -1307,8 +1994,9 @@ __global__ void __launch_bounds__(256, 4) rows_kernel(EnumArgs a) {
     // valid folded points than the fold) is one sector range of the row, and stores also
     // add their per-warp sector counts in closed form.  A warp takes 32 slots at once, one
     // per lane, and each lane walks the runs and stores of its own row.
-    const int64_t q0 = kk * (int64_t)a.chunk_rows;
-    const int64_t q1 = min(q0 + (int64_t)a.chunk_rows, s_c.rows_slot_end[(s_g.levels & 1) ? 3 : 2]);
+    // levels counted in closed form have no slots here
+    const int64_t q0 = ((s_g.foot & 1) || !(s_g.levels & 2) ? s_c.rows_slot_end[2] : 0) + kk * (int64_t)a.chunk_rows;
+    const int64_t q1 = min(q0 + (int64_t)a.chunk_rows, s_c.rows_slot_end[(s_g.levels & 1) && !(s_g.foot & 2) ? 3 : 2]);
     const int L = s_loff[s_g.f_count];
     const int S = s_soff[s_g.f_count] - L;
     const int Mfull = s_ioff[s_g.f_count];
@@ -1549,6 +2237,10 @@ __global__ void __launch_bounds__(256, 4) rows_kernel(EnumArgs a) {
       if (v) atomicAdd(c + dst, v);
     }
   }
+  // then the closed-form items, a warp each, their state in the room of the row walk's access
+  // offsets (every warp has passed the last item's barriers)
+  static_assert(sizeof(FootSmem) * (kRowsThreads / 32) <= sizeof(s_boff) && alignof(FootSmem) <= 16, "FootSmem in s_boff");
+  foot_items(a, reinterpret_cast<FootSmem *>(s_boff)[threadIdx.x >> 5]);
 }
 
 __constant__ int kCountDst[12] = {C_BLK_LS, C_BLK_LL, C_BLK_SS, C_BLK_SL, C_W_LS, C_W_LL,

@@ -263,10 +263,8 @@ static void block_box(int64_t a, int64_t b, const int64_t g[3], int64_t lo[3], i
 static FastDiv make_fastdiv(uint32_t d) {
   FastDiv f;
   f.d = d;
-  f.s = 0;
-  while (((uint64_t)1 << f.s) < d) ++f.s;
+  f.s = d <= 1 ? 0 : 32 - (uint32_t)__builtin_clz(d - 1);
   f.m = (uint32_t)((((uint64_t)1 << 32) * (((uint64_t)1 << f.s) - d)) / d + 1);
-  f.pad = 0;
   return f;
 }
 
@@ -315,17 +313,33 @@ struct CompileArena {
   std::vector<Compiled *> comp;
 };
 
+// The grid row of a merged load run (if all its offsets lie in one) and its x offsets.
+struct RunRow {
+  bool one_row;
+  int64_t dy, dz, dc, dxlo, dxhi;
+};
+
 // What a field compiles to for one folding (independent of domain and block shape):
 // folded access list with byte offsets and first needed folded point, the raw offset
 // range, and per-kv issued-access counts.
 struct FieldFold {
   int status = WS_OK;
   std::vector<DAcc> da;
-  std::vector<DIv> iv;     // merged load runs: without a covering run, covered from another z row, from their own
+  std::vector<DIv> iv;      // merged load runs, then the displacements of the closed form
+  std::vector<RunRow> rr;   // the runs' grid rows
+  // for the row walk (cover_runs): the runs without a covering run, those covered from another z
+  // row, those covered from their own, then the displacements; counts and bounds of this order
+  bool covered = false;
+  std::vector<DIv> iv_cov;
   int32_t n_iv_unc = 0;     // runs without a covering run
   int32_t n_iv_zc = 0;      // runs whose covering run lies in another z row (they come next)
   int16_t cov_dy = 0, cov_dz = 0;   // largest |row displacement| to a covering run
   int16_t cov_dy_y = 0;     // largest |ddy| of the runs covered within their z row (they come last)
+  int32_t n_iv = 0;         // merged load runs
+  int32_t n_dsp[2] = {0, 0};   // displacements of the raw loads / stores
+  int64_t dsp_spread[2] = {0, 0};   // largest less smallest rest of the raw offsets
+  int64_t dsp_y[2] = {0, 0};        // largest less smallest displacement within a plane
+  bool dsp_ok = false;      // the rows have a positive pitch and the displacements fit
   int32_t n_load = 0, n_store = 0;
   __int128 omin = 0, omax = 0;
   int16_t cnt_load[17], cnt_store[17];
@@ -346,6 +360,86 @@ static inline void off_unkey(OffKey q, int64_t o[4]) {
   o[1] = (int64_t)((uint64_t)(q >> 63) & ((1u << 18) - 1)) - (1 << 17);
   o[2] = (int64_t)((uint64_t)(q >> 45) & ((1u << 18) - 1)) - (1 << 17);
   o[3] = (int64_t)((uint64_t)(q >> 4) & (((uint64_t)1 << 41) - 1)) - ((int64_t)1 << 40);
+}
+
+// Displacements of the closed-form footprints (ws_footprint.h): the raw offsets of a field (its
+// folded accesses needed by the first point) as whole rows d of pitch P = elem_bytes * stride_y
+// and a rest of at most P / 2 bytes, one entry per d with the smallest and largest rest.
+static void field_displacements(const ws_field &F, FieldFold &out) {
+  const __int128 P = (__int128)F.elem_bytes * F.stride[1];
+  out.n_dsp[0] = out.n_dsp[1] = 0;
+  out.dsp_spread[0] = out.dsp_spread[1] = 0;
+  out.dsp_ok = P > 0 && P <= ((int64_t)1 << 28);
+  if (!out.dsp_ok) return;
+  const int64_t p = (int64_t)P;
+  const double inv = 1.0 / (double)p;
+  const int64_t ratio = F.stride[2] / F.stride[1];
+  const int32_t q = ratio > 0 && ratio < ((int64_t)1 << 28) && ratio * F.stride[1] == F.stride[2] ? (int32_t)ratio : 0;
+  // (d, c) packed so that unsigned order is lexicographic order: |d| < 2^28, |c| < 2^28
+  static thread_local std::vector<uint64_t> dc;
+  int32_t a = 0;
+  for (int ls = 0; ls < 2; ++ls) {
+    dc.clear();
+    const int32_t end = a + (ls ? out.n_store : out.n_load);
+    int64_t cmin = INT64_MAX, cmax = INT64_MIN;
+    for (; a < end; ++a) {
+      if (out.da[(size_t)a].kmin != 0) continue;
+      const int64_t b = out.da[(size_t)a].boff;
+      // d = round(b / p) but for the product's rounding (|b / p| < 2^28, so c stays within
+      // p / 2 and 16 bytes)
+      const double t = (double)b * inv;
+      if (!(std::fabs(t) < (double)((int64_t)1 << 28) - 1)) {
+        out.dsp_ok = false;
+        break;
+      }
+      const int64_t d = (int64_t)std::floor(t + 0.5), c = b - d * p;
+      cmin = std::min(cmin, c);
+      cmax = std::max(cmax, c);
+      dc.push_back((uint64_t)(d + ((int64_t)1 << 28)) << 32 | (uint64_t)(c + ((int64_t)1 << 30)));
+    }
+    if (!out.dsp_ok) break;
+    if (dc.empty()) continue;
+    std::sort(dc.begin(), dc.end());
+    const size_t at = out.iv.size();
+    out.iv.reserve(at + dc.size());
+    // the smallest displacement within a plane (centred; any value is allowed, it only sets
+    // where the kernel's units begin)
+    int32_t ymin = INT32_MAX, ymax = INT32_MIN;
+    auto d_of = [](uint64_t v) { return (int32_t)(v >> 32) - (1 << 28); };
+    auto c_of = [](uint64_t v) { return (int32_t)((int64_t)(uint32_t)v - ((int64_t)1 << 30)); };
+    for (size_t i = 0; i < dc.size();) {
+      size_t j = i;
+      while (j + 1 < dc.size() && (dc[j + 1] >> 32) == (dc[i] >> 32)) ++j;
+      const DDsp v{d_of(dc[i]), c_of(dc[i]), c_of(dc[j]), 0};
+      int32_t y = v.d;
+      if (q > 0) {
+        y = (y + q / 2) % q;
+        y = (y < 0 ? y + q : y) - q / 2;
+      }
+      ymin = std::min(ymin, y);
+      ymax = std::max(ymax, y);
+      DIv w;
+      memcpy(&w, &v, sizeof(w));
+      out.iv.push_back(w);
+      i = j + 1;
+    }
+    out.n_dsp[ls] = (int32_t)(out.iv.size() - at);
+    out.dsp_spread[ls] = cmax - cmin;
+    out.dsp_y[ls] = (int64_t)ymax - ymin;
+    // the first entry also carries the smallest rest, the second the smallest displacement
+    for (int i = 0; i < std::min(2, out.n_dsp[ls]); ++i) {
+      DDsp v;
+      memcpy(&v, &out.iv[at + (size_t)i], sizeof(v));
+      v.pad = i == 0 ? (int32_t)cmin : ymin;
+      memcpy(&out.iv[at + (size_t)i], &v, sizeof(v));
+    }
+  }
+  // a warp keeps the state of at most 32 x 32 of them
+  if (out.n_dsp[0] > 1024 || out.n_dsp[1] > 1024) out.dsp_ok = false;
+  if (!out.dsp_ok) {
+    out.iv.resize((size_t)out.n_iv);
+    out.n_dsp[0] = out.n_dsp[1] = 0;
+  }
 }
 
 static void compile_field_fold(const ws_field &F, const ws_access *acc, int n_acc, int fold_axis, int fold,
@@ -417,7 +511,7 @@ static void compile_field_fold(const ws_field &F, const ws_access *acc, int n_ac
   out.n_store = (int32_t)sk.size();
   // merged load intervals: sorted load offsets cut wherever two neighbours are more than
   // 32 B apart (a chain of byte addresses with steps of at most 32 B touches every
-  // sector between its ends); for each, the grid row of its offsets and its covering run
+  // sector between its ends); for each, the grid row of its offsets
   {
     struct Ld {
       int64_t b, o[4];   // byte offset; dx dy dz dc
@@ -429,13 +523,11 @@ static void compile_field_fold(const ws_field &F, const ws_access *acc, int n_ac
       off_unkey(lk[(size_t)i], b[(size_t)i].o);
     }
     std::sort(b.begin(), b.end(), [](const Ld &p, const Ld &q) { return p.b < q.b; });
-    struct RunRow {
-      bool one_row;
-      int64_t dy, dz, dc, dxlo, dxhi;
-    };
-    static thread_local std::vector<RunRow> rr;
+    std::vector<RunRow> &rr = out.rr;
     rr.clear();
     out.iv.clear();
+    out.iv_cov.clear();
+    out.covered = false;
     for (size_t i = 0; i < b.size();) {
       size_t j = i;
       while (j + 1 < b.size() && b[j + 1].b - b[j].b <= 32) ++j;
@@ -454,84 +546,9 @@ static void compile_field_fold(const ws_field &F, const ws_access *acc, int n_ac
       rr.push_back(r);
       i = j + 1;
     }
-    // covering runs: order runs by (|dy| + |dz|, dz, dy); a run may be covered by an earlier
-    // one of the same dc whose x offsets contain its own, at a row displacement a thread row
-    // can make (a multiple of the fold along the folding axis); the nearest one is taken
-    const size_t nr = rr.size() <= 512 ? rr.size() : 0;   // bounded host work: no covering beyond 512 runs
-    // The covering run of a run e: among the runs of lower rank (|dy| + |dz|, dz, dy, run)
-    // with the same dc whose x offsets contain its own, at a row displacement a thread row
-    // can make (a multiple of the fold along the folding axis, below 32767 in y and z), the
-    // nearest one, the first of the nearest in run order.  Only one-row runs take part.  They
-    // are visited in rank order, each scanning those before it; the smallest (displacement,
-    // run) score picks the cover.  The rank packs into one integer: |dy|, |dz| <= 65535 + 15
-    // fit 18 bits after a 2^17 bias, their sum 18 bits, the run index (< 512) 9 bits.
-    static thread_local std::vector<int64_t> rk, ry, rz, rres, rxlo, rxhi, rdc, ridx;
-    rk.clear();
-    for (size_t e = 0; e < nr; ++e)
-      if (rr[e].one_row)
-        rk.push_back((int64_t)(((uint64_t)(std::llabs(rr[e].dy) + std::llabs(rr[e].dz)) << 45) |
-                               ((uint64_t)(rr[e].dz + (1 << 17)) << 27) | ((uint64_t)(rr[e].dy + (1 << 17)) << 9) |
-                               (uint64_t)e));
-    std::sort(rk.begin(), rk.end());
-    const size_t no = rk.size();
-    for (auto *v : {&ry, &rz, &rres, &rxlo, &rxhi, &rdc, &ridx}) v->resize(no);
-    const int64_t fm = fold_axis == 0 ? 1 : fold;
-    for (size_t i = 0; i < no; ++i) {
-      const size_t e = (size_t)(rk[i] & 511);
-      const RunRow &r = rr[e];
-      ridx[i] = (int64_t)e;
-      ry[i] = r.dy;
-      rz[i] = r.dz;
-      const int64_t ax = fold_axis == 1 ? r.dy : fold_axis == 2 ? r.dz : 0;
-      rres[i] = ((ax % fm) + fm) % fm;
-      rxlo[i] = r.dxlo;
-      rxhi[i] = r.dxhi;
-      rdc[i] = r.dc;
-    }
-    for (size_t i = 1; i < no; ++i) {
-      const int64_t ye = ry[i], ze = rz[i], re = rres[i], xlo = rxlo[i], xhi = rxhi[i], dce = rdc[i];
-      int64_t best_score = INT64_MAX;
-      for (size_t j = 0; j < i; ++j) {
-        const int64_t ddy = ye - ry[j], ddz = ze - rz[j];
-        const int64_t ay = ddy < 0 ? -ddy : ddy, az = ddz < 0 ? -ddz : ddz;
-        const bool ok = (rdc[j] == dce) & (rxlo[j] <= xlo) & (rxhi[j] >= xhi) & (rres[j] == re) & (ay < 32767) &
-                        (az < 32767);
-        const int64_t score = ok ? (((ay + az) << 9) | ridx[j]) : INT64_MAX;
-        best_score = score < best_score ? score : best_score;
-      }
-      if (best_score != INT64_MAX) {
-        const size_t e = (size_t)ridx[i], best = (size_t)(best_score & 511);
-        out.iv[e].ddy = (int16_t)(rr[e].dy - rr[best].dy);
-        out.iv[e].ddz = (int16_t)(rr[e].dz - rr[best].dz);
-      }
-    }
-    // runs without a covering run first, then those covered from another z row, then those
-    // covered within their own z row (ddz == 0): the row walk takes only the first kind at
-    // rows whose displaced rows all lie inside the level, the first two kinds at rows whose
-    // rows displaced in y alone do, and all runs elsewhere
-    auto kind = [](const DIv &v) { return v.ddy == kNoCover ? 0 : v.ddz != 0 ? 1 : 2; };
-    {
-      static thread_local std::vector<DIv> tmp;
-      tmp.clear();
-      for (int kd = 0; kd < 3; ++kd)
-        for (const DIv &v : out.iv)
-          if (kind(v) == kd) tmp.push_back(v);
-      out.iv.swap(tmp);
-    }
-    out.n_iv_unc = out.n_iv_zc = 0;
-    out.cov_dy = out.cov_dz = out.cov_dy_y = 0;
-    for (const DIv &v : out.iv) {
-      const int kd = kind(v);
-      if (kd == 0) {
-        ++out.n_iv_unc;
-        continue;
-      }
-      if (kd == 1) ++out.n_iv_zc;
-      else out.cov_dy_y = std::max<int16_t>(out.cov_dy_y, (int16_t)std::abs(v.ddy));
-      out.cov_dy = std::max<int16_t>(out.cov_dy, (int16_t)std::abs(v.ddy));
-      out.cov_dz = std::max<int16_t>(out.cov_dz, (int16_t)std::abs(v.ddz));
-    }
   }
+  out.n_iv = (int32_t)out.iv.size();
+  field_displacements(F, out);
   // issued accesses of a thread with kv valid folded points: those with kmin < kv
   int nl = 0, ns = 0;
   for (int kv = 0; kv <= 16; ++kv) {
@@ -541,6 +558,155 @@ static void compile_field_fold(const ws_field &F, const ws_access *acc, int n_ac
       nl += hist[0][kv];
       ns += hist[1][kv];
     }
+  }
+}
+
+// Finds the runs' covering runs.  Only the row walk reads them, so candidates counted in closed form
+// throughout leave them out (finding them is a third of the time a field takes to compile).
+static void cover_runs(int fold_axis, int fold, FieldFold &out) {
+  if (out.covered) return;
+  out.covered = true;
+  const std::vector<RunRow> &rr = out.rr;
+  std::vector<DIv> iv(out.iv.begin(), out.iv.begin() + out.n_iv);
+  // covering runs: order runs by (|dy| + |dz|, dz, dy); a run may be covered by an earlier
+  // one of the same dc whose x offsets contain its own, at a row displacement a thread row
+  // can make (a multiple of the fold along the folding axis); the nearest one is taken
+  const size_t nr = rr.size() <= 512 ? rr.size() : 0;   // bounded host work: no covering beyond 512 runs
+  // The covering run of a run e: among the runs of lower rank (|dy| + |dz|, dz, dy, run)
+  // with the same dc whose x offsets contain its own, at a row displacement a thread row
+  // can make (a multiple of the fold along the folding axis, below 32767 in y and z), the
+  // nearest one, the first of the nearest in run order.  Only one-row runs take part.  They
+  // are visited in rank order, each scanning those before it; the smallest (displacement,
+  // run) score picks the cover.  The rank packs into one integer: |dy|, |dz| <= 65535 + 15
+  // fit 18 bits after a 2^17 bias, their sum 18 bits, the run index (< 512) 9 bits.
+  static thread_local std::vector<int64_t> rk, ry, rz, rres, rxlo, rxhi, rdc, ridx;
+  rk.clear();
+  for (size_t e = 0; e < nr; ++e)
+    if (rr[e].one_row)
+      rk.push_back((int64_t)(((uint64_t)(std::llabs(rr[e].dy) + std::llabs(rr[e].dz)) << 45) |
+                             ((uint64_t)(rr[e].dz + (1 << 17)) << 27) | ((uint64_t)(rr[e].dy + (1 << 17)) << 9) |
+                             (uint64_t)e));
+  std::sort(rk.begin(), rk.end());
+  const size_t no = rk.size();
+  for (auto *v : {&ry, &rz, &rres, &rxlo, &rxhi, &rdc, &ridx}) v->resize(no);
+  const int64_t fm = fold_axis == 0 ? 1 : fold;
+  for (size_t i = 0; i < no; ++i) {
+    const size_t e = (size_t)(rk[i] & 511);
+    const RunRow &r = rr[e];
+    ridx[i] = (int64_t)e;
+    ry[i] = r.dy;
+    rz[i] = r.dz;
+    const int64_t ax = fold_axis == 1 ? r.dy : fold_axis == 2 ? r.dz : 0;
+    rres[i] = ((ax % fm) + fm) % fm;
+    rxlo[i] = r.dxlo;
+    rxhi[i] = r.dxhi;
+    rdc[i] = r.dc;
+  }
+  for (size_t i = 1; i < no; ++i) {
+    const int64_t ye = ry[i], ze = rz[i], re = rres[i], xlo = rxlo[i], xhi = rxhi[i], dce = rdc[i];
+    int64_t best_score = INT64_MAX;
+    for (size_t j = 0; j < i; ++j) {
+      const int64_t ddy = ye - ry[j], ddz = ze - rz[j];
+      const int64_t ay = ddy < 0 ? -ddy : ddy, az = ddz < 0 ? -ddz : ddz;
+      const bool ok = (rdc[j] == dce) & (rxlo[j] <= xlo) & (rxhi[j] >= xhi) & (rres[j] == re) & (ay < 32767) &
+                      (az < 32767);
+      const int64_t score = ok ? (((ay + az) << 9) | ridx[j]) : INT64_MAX;
+      best_score = score < best_score ? score : best_score;
+    }
+    if (best_score != INT64_MAX) {
+      const size_t e = (size_t)ridx[i], best = (size_t)(best_score & 511);
+      iv[e].ddy = (int16_t)(rr[e].dy - rr[best].dy);
+      iv[e].ddz = (int16_t)(rr[e].dz - rr[best].dz);
+    }
+  }
+  // runs without a covering run first, then those covered from another z row, then those
+  // covered within their own z row (ddz == 0): the row walk takes only the first kind at
+  // rows whose displaced rows all lie inside the level, the first two kinds at rows whose
+  // rows displaced in y alone do, and all runs elsewhere
+  auto kind = [](const DIv &v) { return v.ddy == kNoCover ? 0 : v.ddz != 0 ? 1 : 2; };
+  {
+    static thread_local std::vector<DIv> tmp;
+    tmp.clear();
+    for (int kd = 0; kd < 3; ++kd)
+      for (const DIv &v : iv)
+        if (kind(v) == kd) tmp.push_back(v);
+    iv.swap(tmp);
+  }
+  out.n_iv_unc = out.n_iv_zc = 0;
+  out.cov_dy = out.cov_dz = out.cov_dy_y = 0;
+  for (const DIv &v : iv) {
+    const int kd = kind(v);
+    if (kd == 0) {
+      ++out.n_iv_unc;
+      continue;
+    }
+    if (kd == 1) ++out.n_iv_zc;
+    else out.cov_dy_y = std::max<int16_t>(out.cov_dy_y, (int16_t)std::abs(v.ddy));
+    out.cov_dy = std::max<int16_t>(out.cov_dy, (int16_t)std::abs(v.ddy));
+    out.cov_dz = std::max<int16_t>(out.cov_dz, (int16_t)std::abs(v.ddz));
+  }
+  iv.insert(iv.end(), out.iv.begin() + out.n_iv, out.iv.end());
+  out.iv_cov.swap(iv);
+}
+
+// Rows from plane to plane of the field before (a candidate's fields mostly share them); no field
+// has a row stride of 0 here.
+struct RowsPerPlane {
+  int64_t s1 = 0, s2 = 0, q = 0;
+  FastDiv fq = {};
+};
+
+// Levels of a field whose footprints the closed form (ws_footprint.h) counts exactly, df.closed,
+// and its rows from plane to plane, df.q.  pb_lo / pb_hi: point boxes of the block [0] and of the
+// wave and the y / z sets [1]; run_any, shortest_run(level): bound on and length of their shortest
+// runs of x.  Conditions:
+//  * x does not descend, by at most one sector a point; planes are a whole number Q of rows apart
+//    and the level's rows of one plane fit in Q (any Q will do for a level of one plane);
+//  * a row's ranges, from the lowest byte any starts at to the highest any ends at, leave a line
+//    to spare in two pitches, so that they reach no further than the next row's cell;
+//  * within a level's class of runs the ranges overlap or touch: the offsets' rests are spread by
+//    at most the shortest run and one sector.
+template <class Run>
+static void closed_form_ok(const ws_field &F, const FieldFold &ff, int mask, const int64_t pb_lo[2][3],
+                           const int64_t pb_hi[2][3], int64_t n0, int64_t run_any, Run shortest_run,
+                           RowsPerPlane &rows, DField &df) {
+  const int64_t P = (int64_t)F.elem_bytes * F.stride[1], esx = (int64_t)F.elem_bytes * F.stride[0];
+  if (esx < 0 || esx > 32) return;
+  const int64_t spread = std::max(ff.dsp_spread[0], ff.dsp_spread[1]);
+  if (esx * (n0 - 1) + spread + 128 > 2 * P) return;
+  // rows from plane to plane, from the wave's box where the field has one (the block lies in it)
+  const int lq = (mask & 2) ? 1 : 0;
+  const int64_t ny = pb_hi[lq][1] - pb_lo[lq][1] + 1, nz = pb_hi[lq][2] - pb_lo[lq][2] + 1;
+  if (rows.s1 != F.stride[1] || rows.s2 != F.stride[2]) {
+    rows = {F.stride[1], F.stride[2], F.stride[2] / F.stride[1], {}};
+    if (rows.q * F.stride[1] != F.stride[2]) rows.q = 0;
+  }
+  int64_t q = rows.q;
+  const bool planes = q >= ny && q < ((int64_t)1 << 30);   // the displacements' rows within a plane are known
+  if (!planes) {
+    // the level lies in one plane: all its target rows as those of one plane
+    if (nz > 1) return;
+    int64_t dmin = 0, dmax = 0;
+    for (size_t e = (size_t)ff.n_iv; e < ff.iv.size(); ++e) {
+      DDsp d;
+      memcpy(&d, &ff.iv[e], sizeof(d));
+      dmin = std::min<int64_t>(dmin, d.d);
+      dmax = std::max<int64_t>(dmax, d.d);
+    }
+    q = ny + dmax - dmin + 2;
+  }
+  if ((nz - 1) * q + ny >= ((int64_t)1 << 30) || q >= ((int64_t)1 << 30)) return;
+  df.q = (int32_t)q;
+  if (rows.fq.d != (uint32_t)q) rows.fq = make_fastdiv((uint32_t)q);
+  df.fq_m = rows.fq.m;
+  df.fq_s = rows.fq.s;
+  df.y_span_l = (int32_t)(planes ? std::min(ff.dsp_y[0], q) : q);
+  df.y_span_s = (int32_t)(planes ? std::min(ff.dsp_y[1], q) : q);
+  for (int lv = 0; lv < 2; ++lv) {
+    if (!(mask & (1 << lv))) continue;
+    if (spread > esx * (run_any - 1) + 32 && spread > esx * (shortest_run(lv) - 1) + 32) continue;
+    if (lv == 0 && df.words[0] >= ((int64_t)1 << 22)) continue;   // (the block's per-instruction counts)
+    df.closed |= lv == 0 ? 2 : 1;
   }
 }
 
@@ -683,6 +849,7 @@ static uint64_t fold_key(const ws_config &c, int fi) {
   return ((uint64_t)(c.field_off + fi) << 8) | ((uint64_t)c.fold_axis << 5) | (uint64_t)c.fold;
 }
 static const uint64_t kNoShare = ~(uint64_t)0;   // a list that no other descriptor shares
+static const uint64_t kCoveredKey = (uint64_t)1 << 63;   // the list with the covering runs
 
 // Returns WS_OK or a per-candidate error status.  `cache` (may be null) memoizes the
 // per-(field, folding) part across candidates that share fields.
@@ -789,6 +956,8 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     d.fd_b1 = make_fastdiv((uint32_t)c.B[1]);
     d.fd_b2 = make_fastdiv((uint32_t)c.B[2]);
     d.fd_fold = make_fastdiv((uint32_t)c.fold);
+    d.fd_b1f = make_fastdiv((uint32_t)(c.B[1] * fy));
+    d.fd_b2f = make_fastdiv((uint32_t)(c.B[2] * fz));
     const int64_t rng[4][2] = {{s, s + weff}, {y_lo, y_hi}, {z_lo, z_hi}, {rep, rep + 1}};
     int64_t cum = 0;
     for (int lv = 0; lv < 4; ++lv) {
@@ -901,7 +1070,31 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
       }
     }
   };
+  // shortest run of x a level's blocks make in one row: [0] the representative block, [1] the
+  // wave and the y / z sets (no shorter than a block, which settles most fields)
+  const int64_t run_any = std::min<int64_t>(c.B[0], c.N[0] - (int64_t)(g[0] - 1) * c.B[0]);
+  int64_t run_min[2] = {0, 0};
+  RowsPerPlane plane_rows;
+  auto shortest_run = [&](int lv) {
+    auto run = [&](int64_t xa, int64_t xb) { return std::min<int64_t>(xb * c.B[0], c.N[0]) - xa * c.B[0]; };
+    auto shortest = [&](int64_t a, int64_t b) -> int64_t {
+      if (b <= a) return INT64_MAX;
+      if (a / g[0] == (b - 1) / g[0]) return run(a % g[0], (b - 1) % g[0] + 1);
+      return std::min(run(a % g[0], g[0]), run(0, (b - 1) % g[0] + 1));
+    };
+    if (run_min[lv] == 0) {
+      run_min[lv] = lv == 0 ? shortest(rep, rep + 1)
+                            : std::min({shortest(s, s + weff), shortest(y_lo, y_hi), shortest(z_lo, z_hi)});
+      if (lv == 1 && y_hi > y_lo) run_min[1] = std::min(run_min[1], shortest(z_lo, std::min(z_hi, y_lo)));
+    }
+    return run_min[lv];
+  };
+  // A candidate whose levels are all counted in closed form (or by the address walk) needs no
+  // covering runs; a field that the row walk takes turns them on and starts the candidate again.
+  const int kNeedsCovers = INT_MIN;
+  bool covers = false;
   auto emit = [&](const ws_field &F, const FieldFold *ff, int mask, uint64_t key, bool first) -> int {
+    const bool cover = covers && ff->covered;
     DField df;
     memset(&df, 0, sizeof(df));
     df.esize = F.elem_bytes;
@@ -938,6 +1131,11 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     // whole lines, so it has the wave's line count, and only its sectors inside the wave's
     // address range can meet the wave (the row walk clips the z set's ranges to it)
     df.zshift = 0;
+    df.zmove = 0;
+    if (z_is_shifted_wave && (mask & 2) && has_l) {
+      const __int128 by = (__int128)F.elem_bytes * F.stride[2] * c.B[2] * fz;   // the z set lies this far below
+      df.zmove = (uint8_t)(1 + (int)((unsigned __int128)-by & 127));
+    }
     df.zc_lo = 0;
     df.zc_hi = -1;
     if (z_is_shifted_wave && mask == 3 && has_l &&
@@ -971,12 +1169,14 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     // 32-bit offsets, so the wave bitmap must span less than 2^31 bytes
     df.iv = (!df.wide && df.words[1] < ((int64_t)1 << 21) && std::llabs(F.stride[0]) * F.elem_bytes <= 32) ? 1 : 0;
     df.iv_begin = 0;
-    df.n_iv = (int32_t)ff->iv.size();
-    df.n_iv_unc = ff->n_iv_unc;
-    df.n_iv_zc = ff->n_iv_zc;
-    df.cov_dy = ff->cov_dy;
-    df.cov_dz = ff->cov_dz;
-    df.cov_dy_y = ff->cov_dy_y;
+    df.n_iv = ff->n_iv;
+    df.n_iv_unc = cover ? ff->n_iv_unc : ff->n_iv;
+    if (cover) {
+      df.n_iv_zc = ff->n_iv_zc;
+      df.cov_dy = ff->cov_dy;
+      df.cov_dz = ff->cov_dz;
+      df.cov_dy_y = ff->cov_dy_y;
+    }
     // per-instruction store sectors of the row walk add up the row segments of a warp,
     // exact when no two rows of one warp can touch a common sector: their starts lie
     // further apart than a row's byte span plus 31
@@ -997,6 +1197,12 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
           }
         }
     }
+    // closed-form footprints
+    df.n_dsp_l = (int16_t)ff->n_dsp[0];
+    df.n_dsp_s = (int16_t)ff->n_dsp[1];
+    df.closed = 0;
+    df.q = 1;
+    if (ff->dsp_ok) closed_form_ok(F, *ff, mask, pb_lo, pb_hi, c.N[0], run_any, shortest_run, plane_rows, df);
     for (int kv = 0; kv <= 16; ++kv) {
       df.cnt_load[kv] = ff->cnt_load[kv];
       df.cnt_store[kv] = ff->cnt_store[kv];
@@ -1008,22 +1214,27 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     need += page_flag_words(df.words[0], df.words[1]);   // used when the field takes the row walk
     out.f.push_back(df);
     out.acc.insert(out.acc.end(), ff->da.begin(), ff->da.end());
-    out.iv.insert(out.iv.end(), ff->iv.begin(), ff->iv.end());
+    const std::vector<DIv> &iv = cover ? ff->iv_cov : ff->iv;
+    out.iv.insert(out.iv.end(), iv.begin(), iv.end());
     out.acc_off.push_back((int32_t)out.acc.size());
     out.iv_off.push_back((int32_t)out.iv.size());
-    out.fkey.push_back(key);
+    out.fkey.push_back(key != kNoShare && cover ? key | kCoveredKey : key);
     out.need_words.push_back(need);
-    return WS_OK;
+    const int all = (mask & 1 ? 2 : 0) | (mask & 2 ? 1 : 0);
+    return !covers && out.rows_geom_ok && df.iv && df.rows_ok && df.closed != all ? kNeedsCovers : WS_OK;
   };
   // the folded lists of field fi: from the cache when other candidates use the field too,
   // else compiled into `local` (then *own = true: the list is this candidate's alone);
   // tl_fold is this thread's reusable one
   static thread_local FieldFold tl_fold;
+  int local_field = -1;   // the field it holds
   auto fold_of = [&](int fi, FieldFold &local, bool *own) -> FieldFold * {
     const ws_field &F = fld[c.field_off + fi];
     *own = !cache || (field_refs && field_refs[c.field_off + fi] < 2);
     if (*own) {
-      compile_field_fold(F, acc, n_acc, c.fold_axis, c.fold, local);
+      if (local_field != fi) compile_field_fold(F, acc, n_acc, c.fold_axis, c.fold, local);
+      local_field = fi;
+      if (covers && local.status == WS_OK) cover_runs(c.fold_axis, c.fold, local);
       return &local;
     }
     auto it = cache->find(fold_key(c, fi));
@@ -1031,77 +1242,96 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
       it = cache->emplace(fold_key(c, fi), FieldFold()).first;
       compile_field_fold(F, acc, n_acc, c.fold_axis, c.fold, it->second);
     }
+    if (covers && it->second.status == WS_OK) cover_runs(c.fold_axis, c.fold, it->second);
     return &it->second;
   };
-  if (c.address_mode == WS_ADDR_LINEAR) {
-    for (int fi = 0; fi < c.n_field; ++fi) {
-      bool own;
-      FieldFold *ff = fold_of(fi, tl_fold, &own);
-      if (ff->status != WS_OK) return ff->status;
-      const int rc = emit(fld[c.field_off + fi], ff, 3, own ? kNoShare : fold_key(c, fi), fi == 0);
-      if (rc != WS_OK) return rc;
-    }
-  } else {
-    // Multi-dimensional address space (Sec. 4.4.1) for the wave and the y / z sets: a
-    // sector is (innermost bytes / 32, y, z), without the base alignment.  Each field
-    // becomes a block descriptor (linear addresses, as the per-instruction statistics
-    // of the representative block need) and a wave descriptor over a virtual linear
-    // layout in which every (y, z) row is its own 128-byte aligned slab of RS bytes:
-    // virtual address = Xbias + innermost bytes + RS * (y - y0) + PS * (z - z0), so
-    // that virtual sectors and lines are exactly the tuples.  RS and PS are common to
-    // the candidate's fields (equal layouts stay one uniform group).
-    for (int fi = 0; fi < c.n_field; ++fi) {
-      bool own;
-      FieldFold *ff = fold_of(fi, tl_fold, &own);
-      if (ff->status != WS_OK) return ff->status;
-      const int rc = emit(fld[c.field_off + fi], ff, 1, own ? kNoShare : fold_key(c, fi), fi == 0);
-      if (rc != WS_OK) return rc;
-    }
-    __int128 ymin = 0, ymax = 0, zmin = 0, zmax = 0;
-    std::vector<__int128> xlo(c.n_field), xhi(c.n_field);
-    int64_t L = 128;
-    for (int fi = 0; fi < c.n_field; ++fi) {
-      const ws_field &F = fld[c.field_off + fi];
-      int64_t r[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};   // dx dy dz dc ranges of the raw offsets
-      for (int a = 0; a < F.n_access; ++a) {
-        const ws_access &A = acc[F.access_off + a];
-        const int64_t v[4] = {A.dx, A.dy, A.dz, A.dc};
-        for (int q = 0; q < 4; ++q) {
-          r[q][0] = a == 0 ? v[q] : std::min(r[q][0], v[q]);
-          r[q][1] = a == 0 ? v[q] : std::max(r[q][1], v[q]);
-        }
+  auto emit_all = [&]() -> int {
+    if (c.address_mode == WS_ADDR_LINEAR) {
+      for (int fi = 0; fi < c.n_field; ++fi) {
+        bool own;
+        FieldFold *ff = fold_of(fi, tl_fold, &own);
+        if (ff->status != WS_OK) return ff->status;
+        const int rc = emit(fld[c.field_off + fi], ff, 3, own ? kNoShare : fold_key(c, fi), fi == 0);
+        if (rc != WS_OK) return rc;
       }
-      const __int128 x0 = (__int128)F.stride[0] * (pb_lo[1][0] + r[0][0]), x1 = (__int128)F.stride[0] * (pb_hi[1][0] + r[0][1]);
-      xlo[fi] = (__int128)F.elem_bytes * (std::min(x0, x1) + F.const_off + r[3][0]);
-      xhi[fi] = (__int128)F.elem_bytes * (std::max(x0, x1) + F.const_off + r[3][1]);
-      const __int128 y0 = pb_lo[1][1] + r[1][0], y1 = pb_hi[1][1] + r[1][1];
-      const __int128 z0 = pb_lo[1][2] + r[2][0], z1 = pb_hi[1][2] + r[2][1];
-      ymin = fi == 0 ? y0 : std::min(ymin, y0);
-      ymax = fi == 0 ? y1 : std::max(ymax, y1);
-      zmin = fi == 0 ? z0 : std::min(zmin, z0);
-      zmax = fi == 0 ? z1 : std::max(zmax, z1);
-      L = L / std::__gcd(L, (int64_t)F.elem_bytes) * F.elem_bytes;
+    } else {
+      // Multi-dimensional address space (Sec. 4.4.1) for the wave and the y / z sets: a
+      // sector is (innermost bytes / 32, y, z), without the base alignment.  Each field
+      // becomes a block descriptor (linear addresses, as the per-instruction statistics
+      // of the representative block need) and a wave descriptor over a virtual linear
+      // layout in which every (y, z) row is its own 128-byte aligned slab of RS bytes:
+      // virtual address = Xbias + innermost bytes + RS * (y - y0) + PS * (z - z0), so
+      // that virtual sectors and lines are exactly the tuples.  RS and PS are common to
+      // the candidate's fields (equal layouts stay one uniform group).
+      for (int fi = 0; fi < c.n_field; ++fi) {
+        bool own;
+        FieldFold *ff = fold_of(fi, tl_fold, &own);
+        if (ff->status != WS_OK) return ff->status;
+        const int rc = emit(fld[c.field_off + fi], ff, 1, own ? kNoShare : fold_key(c, fi), fi == 0);
+        if (rc != WS_OK) return rc;
+      }
+      __int128 ymin = 0, ymax = 0, zmin = 0, zmax = 0;
+      std::vector<__int128> xlo(c.n_field), xhi(c.n_field);
+      int64_t L = 128;
+      for (int fi = 0; fi < c.n_field; ++fi) {
+        const ws_field &F = fld[c.field_off + fi];
+        int64_t r[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};   // dx dy dz dc ranges of the raw offsets
+        for (int a = 0; a < F.n_access; ++a) {
+          const ws_access &A = acc[F.access_off + a];
+          const int64_t v[4] = {A.dx, A.dy, A.dz, A.dc};
+          for (int q = 0; q < 4; ++q) {
+            r[q][0] = a == 0 ? v[q] : std::min(r[q][0], v[q]);
+            r[q][1] = a == 0 ? v[q] : std::max(r[q][1], v[q]);
+          }
+        }
+        const __int128 x0 = (__int128)F.stride[0] * (pb_lo[1][0] + r[0][0]), x1 = (__int128)F.stride[0] * (pb_hi[1][0] + r[0][1]);
+        xlo[fi] = (__int128)F.elem_bytes * (std::min(x0, x1) + F.const_off + r[3][0]);
+        xhi[fi] = (__int128)F.elem_bytes * (std::max(x0, x1) + F.const_off + r[3][1]);
+        const __int128 y0 = pb_lo[1][1] + r[1][0], y1 = pb_hi[1][1] + r[1][1];
+        const __int128 z0 = pb_lo[1][2] + r[2][0], z1 = pb_hi[1][2] + r[2][1];
+        ymin = fi == 0 ? y0 : std::min(ymin, y0);
+        ymax = fi == 0 ? y1 : std::max(ymax, y1);
+        zmin = fi == 0 ? z0 : std::min(zmin, z0);
+        zmax = fi == 0 ? z1 : std::max(zmax, z1);
+        L = L / std::__gcd(L, (int64_t)F.elem_bytes) * F.elem_bytes;
+      }
+      __int128 row = 0;
+      std::vector<__int128> xbias(c.n_field);
+      for (int fi = 0; fi < c.n_field; ++fi) {
+        xbias[fi] = -floor_div128(xlo[fi], 128) * 128;
+        row = std::max(row, xhi[fi] + xbias[fi] + 1);
+      }
+      const __int128 RS = (row + L - 1) / L * L, PS = RS * (ymax - ymin + 1);
+      if (PS * (zmax - zmin + 1) >= ((__int128)1 << 50)) return WS_ENOMEM;
+      for (int fi = 0; fi < c.n_field; ++fi) {
+        const ws_field &F = fld[c.field_off + fi];
+        ws_field V = F;
+        V.stride[1] = (int64_t)(RS / F.elem_bytes);
+        V.stride[2] = (int64_t)(PS / F.elem_bytes);
+        V.align_bytes = (int64_t)(xbias[fi] - RS * ymin - PS * zmin);
+        compile_field_fold(V, acc, n_acc, c.fold_axis, c.fold, tl_fold);
+        local_field = -1;
+        if (tl_fold.status != WS_OK) return tl_fold.status;
+        if (covers) cover_runs(c.fold_axis, c.fold, tl_fold);
+        const int rc = emit(V, &tl_fold, 2, kNoShare, false);
+        if (rc != WS_OK) return rc;
+      }
     }
-    __int128 row = 0;
-    std::vector<__int128> xbias(c.n_field);
-    for (int fi = 0; fi < c.n_field; ++fi) {
-      xbias[fi] = -floor_div128(xlo[fi], 128) * 128;
-      row = std::max(row, xhi[fi] + xbias[fi] + 1);
-    }
-    const __int128 RS = (row + L - 1) / L * L, PS = RS * (ymax - ymin + 1);
-    if (PS * (zmax - zmin + 1) >= ((__int128)1 << 50)) return WS_ENOMEM;
-    for (int fi = 0; fi < c.n_field; ++fi) {
-      const ws_field &F = fld[c.field_off + fi];
-      ws_field V = F;
-      V.stride[1] = (int64_t)(RS / F.elem_bytes);
-      V.stride[2] = (int64_t)(PS / F.elem_bytes);
-      V.align_bytes = (int64_t)(xbias[fi] - RS * ymin - PS * zmin);
-      compile_field_fold(V, acc, n_acc, c.fold_axis, c.fold, tl_fold);
-      if (tl_fold.status != WS_OK) return tl_fold.status;
-      const int rc = emit(V, &tl_fold, 2, kNoShare, false);
-      if (rc != WS_OK) return rc;
-    }
+    return WS_OK;
+  };
+  int rc = emit_all();
+  if (rc == kNeedsCovers) {
+    covers = true;
+    out.f.clear();
+    out.acc.clear();
+    out.iv.clear();
+    out.acc_off.resize(1);
+    out.iv_off.resize(1);
+    out.fkey.clear();
+    out.need_words.clear();
+    rc = emit_all();
   }
+  if (rc != WS_OK) return rc;
   d.n_field = c.n_field;
   if (!out.f.empty()) block_warp_classes(d, out.f[0].esize, out.f[0].stride, hw, out.cls);
   return WS_OK;
@@ -1186,6 +1416,15 @@ static void default_tuning(ws_tuning &t) {
   if (t.walk != WS_WALK_ADDRESS && t.walk != WS_WALK_SEGMENT) t.walk = WS_WALK_INTERVAL;
 }
 
+// Closed-form items are shares of a field of foot_unit estimated warp instructions (ClosedFormCost),
+// at most kFootParts of them: three for every resident warp, or two while those stay below
+// kFootUnitSmall (an item's set-up, some 20 us with the instructions' fetch, then costs more than
+// evenness gives: 76 25-point candidates 73 -> 67 us with two, 40 served ones 96 -> 84; 755 of
+// the former 0.230 -> 0.256 ms, which keep three), and at most kFootUnitMax (4,000 mixed
+// candidates 1.90 ms, with 8000 2.13).
+static constexpr int64_t kFootUnitMin = 1000, kFootUnitSmall = 10000, kFootUnitMax = 32000, kFootParts = 64,
+                         kFootPerWarp = 3;
+
 // Numbers work items and cuts passes for the current tuning.
 // Runs fn(lo, hi) over [0, n) in chunks on the host pool (defined with the pool below).
 static void parallel_chunks(int64_t n, int64_t chunk, const std::function<void(int64_t, int64_t)> &fn);
@@ -1215,6 +1454,7 @@ void ws_plan::layout() {
       DGroup &G = hgrp[(size_t)g];
       G.iv = grp_iv_ok[(size_t)g] && tune.walk != WS_WALK_ADDRESS;
       G.rows = grp_rows_ok[(size_t)g] && tune.walk == WS_WALK_INTERVAL;
+      G.foot = G.rows ? grp_foot_ok[(size_t)g] & ((G.levels & 1 ? 2 : 0) | (G.levels & 2 ? 1 : 0)) : 0;
       // the row walk builds the block bitmaps, so the block path counts one warp per
       // class; otherwise it inserts every warp
       const bool classes = G.rows && (G.levels & 1) && grp_classes[(size_t)g].n > 0;
@@ -1239,28 +1479,60 @@ void ws_plan::layout() {
   for (int64_t v : gneed) max_need = std::max(max_need, v);
   int64_t cap = scratch_words;
   if (tune.pass_mb > 0) cap = std::min(cap, std::max(max_need, (int64_t)tune.pass_mb << 18));
+  // row slots a group's row walk visits: levels counted in closed form have none
+  auto row_slots = [&](int g) -> int64_t {
+    const DGroup &G = hgrp[(size_t)g];
+    if (!G.rows) return 0;
+    const int64_t blk = grp_blk_slots[(size_t)g], all = grp_slots[(size_t)g];
+    return ((G.foot & 1) || !(G.levels & 2) ? 0 : all - blk) + (G.foot & 2 ? 0 : blk);
+  };
   // row slots per row-walk item: 256 (one 32-slot batch for each of a CTA's eight warps),
-  // doubled up to 1024 while every resident row-walk CTA (four per SM; a dry run without a
-  // device assumes 152 SMs) still gets at least 32 items.  Larger items cost less per slot
+  // doubled up to 1024 while four row-walk CTAs per SM (a dry run without a device assumes
+  // 152 SMs) would still get at least 32 items each.  Larger items cost less per slot
   // (the mixed set's row walk 12.8 -> 12.0 ms at 1024), the small sweeps need the finer
   // split to balance (LBM 1.33 -> 1.51 ms at 1024)
   {
     int64_t slots = 0;
     for (int g = 0; g < ng; ++g)
-      if (hgrp[(size_t)g].rows) slots += grp_slots[(size_t)g];
+      slots += row_slots(g);
     const int64_t ctas = 4 * (int64_t)(ctx ? ctx->sm_count : 152);
     rows_chunk = 256;
     while (!plain_layout && rows_chunk < 1024 && slots / (2 * rows_chunk) >= 32 * ctas) rows_chunk *= 2;
   }
   block_pairs = plain_layout ? kPlainBlockPairs : kBlockPairs;
   count_pack = plain_layout ? 1 : kCountItemUnits;
+  // closed-form items: a field's units are shared out among parts of foot_unit estimated warp
+  // instructions (kFootPerWarp and its neighbours; two CTAs of eight warps are resident per SM),
+  // without exceeding the owner-table entries the descriptor estimate allowed for
+  int64_t foot_unit = kFootUnitMin;
+  {
+    const int64_t warps = 16 * (int64_t)(ctx ? ctx->sm_count : 152);
+    int64_t cost = 0, fields = 0;
+    for (int g = 0; g < ng; ++g)
+      if (hgrp[(size_t)g].foot) {
+        const int n = __builtin_popcount(hgrp[(size_t)g].foot_fields);
+        cost += grp_foot_cost[(size_t)g] * n;
+        fields += n;
+      }
+    if (!plain_layout) {
+      foot_unit = std::max({foot_unit, std::min(cost / (kFootPerWarp * warps), kFootUnitMax),
+                            std::min(cost / ((kFootPerWarp - 1) * warps), kFootUnitSmall)});
+    }
+    if (own_budget > 0) foot_unit = std::max(foot_unit, cost / std::max<int64_t>(1, own_budget / 2));
+    foot_chunk = (int32_t)std::max<int64_t>(1, std::min<int64_t>(8, fields / (64 * warps)));
+    if (plain_layout) foot_chunk = 1;
+    int foot_groups = 0;
+    for (int g = 0; g < ng; ++g) foot_groups += hgrp[(size_t)g].foot != 0;
+    const int64_t share = 4 * warps / std::max<int64_t>(1, plain_layout ? 1 : foot_groups);
+    foot_stat = (int32_t)std::max<int64_t>(1, std::min<int64_t>(8, share));
+  }
   // passes (a group starts a new one when its words would overflow the capacity), each
   // group's first scratch word in its pass, and the enumeration and row-walk items: the
   // representative block (exact path) in chunks of (modelled warp, instruction) pairs; then
   // chunks of the remaining modelled warps, or, for the row walk, chunks of row slots
   std::vector<int64_t> gbase((size_t)ng, 0);
   std::vector<int32_t> gpass((size_t)ng, 0);
-  int64_t items = 0, ritems = 0;
+  int64_t items = 0, ritems = 0, fitems = 0;
   {
     DPass cur;
     memset(&cur, 0, sizeof(cur));
@@ -1272,11 +1544,13 @@ void ws_plan::layout() {
         cur.grp_hi = g;
         cur.item_hi = items;
         cur.ritem_hi = ritems;
+        cur.fitem_hi = fitems;
         cur.words = used;
         passes.push_back(cur);
         memset(&cur, 0, sizeof(cur));
         cur.item_lo = items;
         cur.ritem_lo = ritems;
+        cur.fitem_lo = fitems;
         cur.cf_lo = G.f_begin;
         cur.grp_lo = g;
         used = 0;
@@ -1289,15 +1563,40 @@ void ws_plan::layout() {
       G.n0_items = (G.levels & 1) ? (int32_t)std::max<int64_t>(1, ceil_div((int64_t)G.n_rep * G.acc_count, block_pairs))
                                   : 0;
       items += G.n0_items;
-      if (G.rows) ritems += ceil_div(grp_slots[(size_t)g], chunk_rows());
+      G.fitem_begin = fitems;
+      G.f_parts = G.foot ? (int32_t)std::max<int64_t>(1, std::min<int64_t>(kFootParts, grp_foot_cost[(size_t)g] / foot_unit)) : 0;
+      fitems += (int64_t)__builtin_popcount(G.foot_fields) * G.f_parts;
+      if (G.rows) ritems += ceil_div(row_slots(g), chunk_rows());
       else if (G.levels & 2) items += ceil_div(G.mw_end - G.mw_block, tune.chunk_warps);
     }
     cur.cf_hi = (int)hfld.size();
     cur.grp_hi = ng;
     cur.item_hi = items;
     cur.ritem_hi = ritems;
+    cur.fitem_hi = fitems;
     cur.words = used;
     if (ng > 0) passes.push_back(cur);
+  }
+  // the warps take the closed-form items in order: those of the longest parts first (by powers of
+  // two), so that none of them is left for the end
+  if (!plain_layout) {
+    auto bucket = [&](int g) {
+      const int64_t c = grp_foot_cost[(size_t)g] / std::max(1, hgrp[(size_t)g].f_parts);
+      return c > 0 ? __builtin_clzll((unsigned long long)c) : 64;
+    };
+    for (const DPass &P : passes) {
+      int64_t at[66] = {0};
+      for (int g = P.grp_lo; g < P.grp_hi; ++g)
+        at[bucket(g) + 1] += (int64_t)__builtin_popcount(hgrp[(size_t)g].foot_fields) * hgrp[(size_t)g].f_parts;
+      at[0] = P.fitem_lo;
+      for (int b = 0; b < 65; ++b) at[b + 1] += at[b];
+      for (int g = P.grp_lo; g < P.grp_hi; ++g) {
+        DGroup &G = hgrp[(size_t)g];
+        int64_t &next = at[bucket(g)];
+        G.fitem_begin = next;
+        next += (int64_t)__builtin_popcount(G.foot_fields) * G.f_parts;
+      }
+    }
   }
   // counting: units (field, chunk) packed into items of consecutive units of one candidate
   // and pass (at most kCountMaxPages pages and count_pack units), so that the many small
@@ -1311,11 +1610,12 @@ void ws_plan::layout() {
       seg_start.push_back(g);
   const int64_t nseg = (int64_t)seg_start.size();
   seg_start.push_back(ng);
-  std::vector<int64_t> seg_items((size_t)nseg + 1, 0), seg_units((size_t)nseg + 1, 0);
+  std::vector<int64_t> seg_items((size_t)nseg + 1, 0), seg_units((size_t)nseg + 1, 0), seg_acct((size_t)nseg + 1, 0);
   std::vector<int32_t> citem_unit_, cunits_;
   auto pack = [&](int64_t sg, bool write, int64_t item0, int64_t unit0) {
     bool open = false;
     int64_t n_items = 0, n_units = 0, pages_in = 0, units_in = 0;
+    int64_t a_items = 0, a_pages = 0, a_units = 0;   // the same with the units the closed form makes needless
     for (int g = seg_start[(size_t)sg]; g < seg_start[(size_t)sg + 1]; ++g) {
       const DGroup &G = hgrp[(size_t)g];
       int64_t o = gbase[(size_t)g];
@@ -1344,7 +1644,15 @@ void ws_plan::layout() {
           f.item_begin = G.item_begin;
           f.citem_begin = item0 + n_items - (open ? 1 : 0);
         }
+        const int64_t kb = ceil_div(f.words[0], G.rows ? (int64_t)kPagedChunkWords : (int64_t)tune.count_words);
         for_count_units(f, G.rows != 0, tune.count_words, [&](int64_t u, int64_t pages) {
+          if (a_items == 0 || a_pages + pages > kCountMaxPages || a_units == count_pack) {
+            ++a_items;
+            a_pages = a_units = 0;
+          }
+          a_pages += pages;
+          ++a_units;
+          if (G.foot & (u < kb ? 2 : 1)) return;
           if (!open || pages_in + pages > kCountMaxPages || units_in == count_pack) {
             if (write) citem_unit_[(size_t)(item0 + n_items)] = (int32_t)(unit0 + n_units);
             ++n_items;
@@ -1362,6 +1670,7 @@ void ws_plan::layout() {
       }
     }
     seg_items[(size_t)sg] = n_items;
+    seg_acct[(size_t)sg] = a_items;
     seg_units[(size_t)sg] = n_units;
   };
   parallel_chunks(nseg, 64, [&](int64_t lo, int64_t hi) {
@@ -1373,6 +1682,8 @@ void ws_plan::layout() {
     seg_unit0[(size_t)sg + 1] = seg_unit0[(size_t)sg] + seg_units[(size_t)sg];
   }
   const int64_t citems = seg_item0[(size_t)nseg], units = seg_unit0[(size_t)nseg];
+  citems_accounted = 0;
+  for (int64_t sg = 0; sg < nseg; ++sg) citems_accounted += seg_acct[(size_t)sg];
   citem_unit_.assign((size_t)citems, 0);
   cunits_.assign((size_t)(2 * units), 0);
   parallel_chunks(nseg, 64, [&](int64_t lo, int64_t hi) {
@@ -1390,9 +1701,10 @@ void ws_plan::layout() {
   item_begin_end = items;
   ritem_begin_end = ritems;
   citem_begin_end = citems;
-  // owners of the items: [enumeration | row walk], then the counting items' first units
-  // (with an end), then the counting units as (field, chunk) pairs
-  own.resize((size_t)(items + ritems + citems + 1) + cunits_.size());
+  fitem_begin_end = fitems;
+  // owners of the items: [enumeration | row walk | closed form], then the counting items' first
+  // units (with an end), then the counting units as (field, chunk) pairs
+  own.resize((size_t)(items + ritems + fitems + citems + 1) + cunits_.size());
   parallel_chunks(ng, 1024, [&](int64_t lo, int64_t hi) {
     for (int64_t g = lo; g < hi; ++g) {
       const DGroup &G = hgrp[(size_t)g];
@@ -1400,11 +1712,14 @@ void ws_plan::layout() {
       const int64_t r1 = g + 1 < ng ? hgrp[(size_t)g + 1].ritem_begin : ritems;
       std::fill(own.begin() + G.item_begin, own.begin() + e1, (int32_t)g);
       std::fill(own.begin() + items + G.ritem_begin, own.begin() + items + r1, (int32_t)g);
+      std::fill_n(own.begin() + items + ritems + G.fitem_begin, (int64_t)__builtin_popcount(G.foot_fields) * G.f_parts,
+                  (int32_t)g);
     }
   });
-  std::copy(citem_unit_.begin(), citem_unit_.end(), own.begin() + items + ritems);
-  own[(size_t)(items + ritems + citems)] = (int32_t)units;
-  std::copy(cunits_.begin(), cunits_.end(), own.begin() + items + ritems + citems + 1);
+  const int64_t at = items + ritems + fitems;
+  std::copy(citem_unit_.begin(), citem_unit_.end(), own.begin() + at);
+  own[(size_t)(at + citems)] = (int32_t)units;
+  std::copy(cunits_.begin(), cunits_.end(), own.begin() + at + citems + 1);
 }
 
 int ws_plan::upload_fields(cudaStream_t st) {
@@ -1445,12 +1760,14 @@ int ws_plan::bank_shift() const {
   return sh;
 }
 
-int ws_plan::grid_rows(int64_t items) const {
+// CTAs of the row-walk kernel: one per row-walk item, one per eight warps' closed-form items.
+int ws_plan::grid_rows(int64_t items, int64_t fitems) const {
   int occ = 1;
   rows_occupancy(iv_cap, &occ);
   if (tune.ctas_per_sm > 0) occ = std::min(occ, tune.ctas_per_sm);
   occ = std::max(occ, 1);
   int64_t g = (int64_t)ctx->sm_count * occ;
+  items = std::max(items, ceil_div(fitems * (1 + foot_stat), (int64_t)foot_chunk * (kRowsThreads / 32)));
   g = std::min<int64_t>(g, std::max<int64_t>(items, 1));
   return (int)g;
 }
@@ -1489,12 +1806,20 @@ int ws_plan::enqueue(cudaStream_t st, std::vector<cudaEvent_t> *ev, ws_profile *
     ea.iv_cap = iv_cap;
     ea.scratch = (uint32_t *)dev(d_scratch);
     ea.counters = (int64_t *)((char *)dev(d_counters) + grab_bytes);
-    ea.grab = (unsigned long long *)dev(d_counters) + 3 * p;
+    ea.grab = (unsigned long long *)dev(d_counters) + 4 * p;
     ea.rgrab = ea.grab + 1;
+    ea.fgrab = ea.grab + 3;
     ea.own_enum = (const int32_t *)dev(d_own);
     ea.own_rows = ea.own_enum + item_begin_end;
+    ea.own_foot = ea.own_rows + ritem_begin_end;
+    ea.fchunk = foot_chunk;
+    ea.fstat = foot_stat;
     ea.ritem_lo = P.ritem_lo;
     ea.ritem_hi = P.ritem_hi;
+    ea.fitem_lo = P.fitem_lo;
+    ea.fitem_hi = P.fitem_hi;
+    ea.grp_lo = P.grp_lo;
+    ea.grp_hi = P.grp_hi;
     ea.item_lo = P.item_lo;
     ea.item_hi = P.item_hi;
     ea.chunk = tune.chunk_warps;
@@ -1509,14 +1834,14 @@ int ws_plan::enqueue(cudaStream_t st, std::vector<cudaEvent_t> *ev, ws_profile *
       ++launches;
     }
     if ((rc = mark(1 + 3 * (int)p)) != WS_OK) return rc;
-    if (P.ritem_hi > P.ritem_lo) {
-      CU(launch_rows(ea, grid_rows(P.ritem_hi - P.ritem_lo), st));
+    if (P.ritem_hi > P.ritem_lo || P.fitem_hi > P.fitem_lo) {
+      CU(launch_rows(ea, grid_rows(P.ritem_hi - P.ritem_lo, P.fitem_hi - P.fitem_lo), st));
       ++launches;
     }
     if ((rc = mark(2 + 3 * (int)p)) != WS_OK) return rc;
     CountArgs ca;
     ca.fld = ea.fld;
-    ca.item_unit = ea.own_rows + ritem_begin_end;
+    ca.item_unit = ea.own_foot + fitem_begin_end;
     ca.units = ca.item_unit + citem_begin_end + 1;
     ca.scratch = ea.scratch;
     ca.counters = ea.counters;
@@ -1592,7 +1917,8 @@ int ws_plan::run_plain_launches(cudaStream_t st) {
       const int cf_lo = hgrp[glo].f_begin, cf_hi = hgrp[ghi - 1].f_begin + hgrp[ghi - 1].f_count;
       const int64_t ct_lo = hfld[cf_lo].citem_begin, ct_hi = cf_hi < nf ? hfld[cf_hi].citem_begin : citem_begin_end;
       const int64_t rt_lo = hgrp[glo].ritem_begin, rt_hi = ghi < ng ? hgrp[ghi].ritem_begin : ritem_begin_end;
-      CU(cudaMemsetAsync(grab, 0, 3 * sizeof(unsigned long long), st));
+      const int64_t ft_lo = hgrp[glo].fitem_begin, ft_hi = ghi < ng ? hgrp[ghi].fitem_begin : fitem_begin_end;
+      CU(cudaMemsetAsync(grab, 0, 4 * sizeof(unsigned long long), st));
       EnumArgs ea;
       ea.cfg = (const DCfg *)dev(d_cfg);
       ea.fld = (const DField *)dev(d_fld);
@@ -1604,12 +1930,20 @@ int ws_plan::run_plain_launches(cudaStream_t st) {
       ea.counters = counters;
       ea.grab = grab;
       ea.rgrab = grab + 1;
+      ea.fgrab = grab + 3;
       ea.own_enum = (const int32_t *)dev(d_own);
       ea.own_rows = ea.own_enum + item_begin_end;
+      ea.own_foot = ea.own_rows + ritem_begin_end;
+      ea.fchunk = foot_chunk;
+      ea.fstat = foot_stat;
       ea.item_lo = it_lo;
       ea.item_hi = it_hi;
       ea.ritem_lo = rt_lo;
       ea.ritem_hi = rt_hi;
+      ea.fitem_lo = ft_lo;
+      ea.fitem_hi = ft_hi;
+      ea.grp_lo = glo;
+      ea.grp_hi = ghi;
       ea.chunk = tune.chunk_warps;
       ea.chunk_rows = chunk_rows();
       ea.banks = hw.banks;
@@ -1618,10 +1952,10 @@ int ws_plan::run_plain_launches(cudaStream_t st) {
       ea.bank_shift = bank_shift();
       ea.block_pairs = block_pairs;
       if (it_hi > it_lo) CU(launch_enum(ea, grid_for(tune.enum_threads, it_hi - it_lo, false), tune.enum_threads, st));
-      if (rt_hi > rt_lo) CU(launch_rows(ea, grid_rows(rt_hi - rt_lo), st));
+      if (rt_hi > rt_lo || ft_hi > ft_lo) CU(launch_rows(ea, grid_rows(rt_hi - rt_lo, ft_hi - ft_lo), st));
       CountArgs ca;
       ca.fld = ea.fld;
-      ca.item_unit = ea.own_rows + ritem_begin_end;
+      ca.item_unit = ea.own_foot + fitem_begin_end;
       ca.units = ca.item_unit + citem_begin_end + 1;
       ca.scratch = ea.scratch;
       ca.counters = counters;
@@ -1939,7 +2273,10 @@ static void compile_all(const ws_config *cfgs, int n_cfg, const ws_field *fld, i
         const size_t cr = 256;   // the smallest row-walk item
         for (size_t k = 0; k < cc.f.size(); ++k) {
           const int64_t nacc = cc.acc_off[k + 1] - cc.acc_off[k], niv = cc.iv_off[k + 1] - cc.iv_off[k];
-          cc.dsc_bytes += sizeof(DField) + sizeof(DGroup) + (size_t)nacc * sizeof(DAcc) + (size_t)niv * sizeof(DIv);
+          // the displacements of the closed form are left to the estimate's slack (a group per
+          // field, owner-table entries of items the closed form does not make) and headroom
+          cc.dsc_bytes += sizeof(DField) + sizeof(DGroup) + (size_t)nacc * sizeof(DAcc) +
+                          (size_t)cc.f[k].n_iv * sizeof(DIv);
           cc.need_sum += (size_t)cc.need_words[k] * 4;
           cc.need_max = std::max(cc.need_max, (size_t)cc.need_words[k] * 4);
           // at most one enumeration item per chunk of modelled warps and one row-walk item per
@@ -1969,7 +2306,7 @@ int ws::plan_requirements(const ws_config *cfgs, int n_cfg, const ws_field *fld,
     if (compile_config(cfgs[i], fld, n_fld, acc, n_acc, *hw, cc, &cache) != WS_OK) continue;
     for (size_t k = 0; k < cc.f.size(); ++k) {
       dsc += sizeof(DField) + sizeof(DGroup) + (size_t)(cc.acc_off[k + 1] - cc.acc_off[k]) * sizeof(DAcc) +
-             (size_t)(cc.iv_off[k + 1] - cc.iv_off[k]) * sizeof(DIv);
+             (size_t)cc.f[k].n_iv * sizeof(DIv);
       scr += (size_t)cc.need_words[k] * 4;
       mf = std::max(mf, (size_t)cc.need_words[k] * 4);
     }
@@ -1991,21 +2328,98 @@ struct HostDesc {
   size_t scratch = 0, desc_bytes = 0;
 };
 
-// Field groups of candidate i (fields already in p->hfld): consecutive fields bounded by
-// the shared-memory staging (fields, folded accesses) and by what one pass of scratch
-// holds; appended to `go` with the per-group walk decisions.
+// Estimates the warp instructions of a field's closed-form items (ws_kernels.cu, foot_task): units of
+// repeated planes (few where blocks are deep: the planes within reach of a slab's ends one by
+// one, the rest together), windows of each, displacements looked up in each.  Against a count of
+// the operations of four sets of candidates the heaviest twentieth of the fields is within a
+// factor of two.
+struct ClosedFormCost {
+  // of the wave, the z set and the block: planes, slabs, windows of a unit
+  float planes[3], slabs[3], windows[3];
+  explicit ClosedFormCost(const DCfg &dc) {
+    const int64_t b2f = dc.B[2] * (dc.fold_axis == 2 ? dc.fold : 1), b1f = dc.B[1] * (dc.fold_axis == 1 ? dc.fold : 1);
+    const double per_row = 1.0 / (double)dc.g[0], per_slab = per_row / (double)dc.g[1];
+    const int64_t range[3][2] = {{dc.s, dc.s + dc.weff}, {dc.z_lo, dc.z_hi}, {dc.rep, dc.rep + 1}};
+    for (int l = 0; l < 3; ++l) {
+      planes[l] = slabs[l] = windows[l] = 0;
+      const int64_t lo = range[l][0], hi = range[l][1];
+      if (hi <= lo) continue;
+      const double n = (double)((int64_t)((double)(hi - 1) * per_slab) - (int64_t)((double)lo * per_slab) + 1);
+      const double by = (double)((int64_t)((double)(hi - 1) * per_row) - (int64_t)((double)lo * per_row) + 1);
+      const double rows = n > 1 ? dc.N[1] : std::min<double>(by * (double)b1f, dc.N[1]);
+      planes[l] = (float)std::min<double>(n * (double)b2f, dc.N[2]);
+      slabs[l] = (float)n;
+      windows[l] = std::min(1 + (float)rows / 32, 4.0f);
+    }
+  }
+  // of the heaviest of a group's fields: nd and reach, the largest numbers of load displacements
+  // and of planes they span
+  float of(int levels, bool stores, int nd, float reach, bool z_moved) const {
+    float cost = stores ? 3500 : 500;
+    if (nd == 0) return cost;
+    const float each = 700 + 50.0f * (float)std::min(nd, 24);
+    auto level = [&](int l) {
+      return std::min(planes[l] + reach, slabs[l] * (reach + 2) + reach + 1) * windows[l] * each;
+    };
+    if (levels & 2) cost += level(0) + (z_moved ? 0 : level(1));
+    return levels & 1 ? cost + 0.6f * level(2) : cost;
+  }
+};
+
 struct GroupOut {
   std::vector<DGroup> g;
-  std::vector<char> iv_ok, rows_ok;
-  std::vector<int64_t> slots, winstr;
+  std::vector<char> iv_ok, rows_ok, foot_ok;
+  std::vector<int64_t> slots, blk_slots, winstr, foot_cost;
   std::vector<WarpClasses> cls;
   int32_t iv_cap = 0;
 };
 
-static void build_groups(const Plan *p, int i, const Compiled &cc, const ws_hw &hw, GroupOut &go) {
+// Fields of a group whose loads (stores) are another one's moved by a whole number of lines have
+// its footprint counts: the first of each such class is counted with the class's size (mult_l,
+// mult_s), the others not at all.  A field's ranges are the group's common runs moved by
+// base + P * d + [clo, chi] over its displacements, so two lists agree up to a move when the
+// starts differ by one constant throughout and the widths are the same.
+static void count_moved_copies(Plan *p, DGroup &G, const Compiled &cc, int a) {
+  G.foot_fields = 0;
+  const DField &f0 = p->hfld[G.f_begin];
+  const int64_t P = (int64_t)f0.esize * f0.stride[1];
+  auto list = [&](int k, int ls) {
+    const DField &f = p->hfld[G.f_begin + k];
+    return reinterpret_cast<const DDsp *>(cc.iv.data() + cc.iv_off[G.f_begin + k - a] + f.n_iv) + (ls ? f.n_dsp_l : 0);
+  };
+  auto moved = [&](int j, int k, int ls, int nd) {
+    const DDsp *e = list(j, ls), *d = list(k, ls);
+    const int64_t by = P * ((int64_t)d[0].d - e[0].d) + d[0].clo - e[0].clo;
+    if ((by + p->hfld[G.f_begin + k].base - p->hfld[G.f_begin + j].base) & 127) return false;
+    for (int q = 0; q < nd; ++q)
+      if (P * ((int64_t)d[q].d - e[q].d) + d[q].clo - e[q].clo != by || d[q].chi - d[q].clo != e[q].chi - e[q].clo)
+        return false;
+    return true;
+  };
+  for (int k = 0; k < G.f_count; ++k) {
+    DField &f = p->hfld[G.f_begin + k];
+    f.mult_l = f.n_dsp_l > 0;
+    f.mult_s = f.n_dsp_s > 0;
+    for (int j = 0; j < k && f.mult_l; ++j) {
+      DField &g = p->hfld[G.f_begin + j];
+      if (g.mult_l && g.n_dsp_l == f.n_dsp_l && moved(j, k, 0, f.n_dsp_l)) ++g.mult_l, f.mult_l = 0;
+    }
+    for (int j = 0; j < k && f.mult_s; ++j) {
+      DField &g = p->hfld[G.f_begin + j];
+      if (g.mult_s && g.n_dsp_s == f.n_dsp_s && moved(j, k, 1, f.n_dsp_s)) ++g.mult_s, f.mult_s = 0;
+    }
+    if (f.mult_l || f.mult_s) G.foot_fields |= 1u << k;
+  }
+}
+
+// Field groups of candidate i (fields already in p->hfld): consecutive fields bounded by
+// the shared-memory staging (fields, folded accesses) and by what one pass of scratch
+// holds; appended to `go` with the per-group walk decisions.
+static void build_groups(Plan *p, int i, const Compiled &cc, const ws_hw &hw, GroupOut &go) {
   const int a = p->cfg_cf_begin[i], b = p->cfg_cf_begin[i + 1];
   int k = a;
   bool wave_seen = false;
+  const ClosedFormCost cost_of(cc.d);
   while (k < b) {
     DGroup G;
     memset(&G, 0, sizeof(G));
@@ -2047,7 +2461,7 @@ static void build_groups(const Plan *p, int i, const Compiled &cc, const ws_hw &
     G.iv = G.iv && G.uniform;
     if (G.iv) go.iv_cap = std::max(go.iv_cap, G.n_iv);
     // row walk: interval groups whose store counts add up per row segment
-    bool rows = G.iv && cc.rows_geom_ok && (G.levels & 2);
+    bool rows = G.iv && cc.rows_geom_ok;
     int64_t instr_w = 0, instr_yz = 0;
     for (int q = G.f_begin; q < G.f_begin + G.f_count; ++q) {
       rows = rows && p->hfld[q].rows_ok;
@@ -2056,13 +2470,37 @@ static void build_groups(const Plan *p, int i, const Compiled &cc, const ws_hw &
     }
     const DCfg &dc = cc.d;
     go.iv_ok.push_back((char)G.iv);
-    go.rows_ok.push_back((char)rows);
+    // closed-form footprints where every field allows them (a level the group does not serve
+    // counts as one); a group whose levels all do needs no bitmaps, however large they would be
+    int foot = cc.rows_geom_ok ? 3 : 0;
+    int nd = 0;
+    float reach = 0;
+    bool stores = false, z_moved = true;
+    for (int q = G.f_begin; q < G.f_begin + G.f_count; ++q) {
+      const DField &f = p->hfld[q], &f0 = p->hfld[G.f_begin];
+      const bool same = f.esize == f0.esize && f.stride[0] == f0.stride[0] && f.stride[1] == f0.stride[1] &&
+                        f.stride[2] == f0.stride[2];
+      foot &= same && f.rows_ok ? f.closed | (~G.levels & 1 ? 2 : 0) | (~G.levels & 2 ? 1 : 0) : 0;
+      const DDsp *d = reinterpret_cast<const DDsp *>(cc.iv.data() + cc.iv_off[q - a] + f.n_iv);
+      stores = stores || f.n_dsp_s > 0;
+      if (f.n_dsp_l > 0) {
+        nd = std::max(nd, (int)f.n_dsp_l);
+        reach = std::max(reach, (float)((int64_t)d[f.n_dsp_l - 1].d - d[0].d) / (float)std::max(1, f.q));
+        z_moved = z_moved && f.zmove;
+      }
+    }
+    if (!rows && foot != 3) foot = 0;
+    if (foot) count_moved_copies(p, G, cc, a);
+    go.rows_ok.push_back((char)(rows || foot == 3));
+    go.foot_ok.push_back((char)foot);
+    go.foot_cost.push_back(foot ? (int64_t)cost_of.of(G.levels, stores, nd, reach, z_moved) : 0);
     // with the block level when the group also serves the representative block
     go.slots.push_back(dc.rows_slot_end[(G.levels & 1) ? 3 : 2]);
+    go.blk_slots.push_back((G.levels & 1) ? dc.rows_slot_end[3] - dc.rows_slot_end[2] : 0);
     {
       const DField &f0 = p->hfld[G.f_begin], &c0 = p->hfld[a];
       WarpClasses wc;
-      if (rows && (G.levels & 1)) {
+      if ((rows || foot == 3) && (G.levels & 1)) {
         if (f0.esize == c0.esize && f0.stride[0] == c0.stride[0] && f0.stride[1] == c0.stride[1] &&
             f0.stride[2] == c0.stride[2])
           wc = cc.cls;
@@ -2071,7 +2509,9 @@ static void build_groups(const Plan *p, int i, const Compiled &cc, const ws_hw &
       }
       go.cls.push_back(wc);
     }
-    go.winstr.push_back((cc.lvl_blocks[0] * instr_w + (cc.lvl_blocks[1] + cc.lvl_blocks[2]) * instr_yz) * dc.wpb);
+    go.winstr.push_back(G.levels & 2
+                            ? (cc.lvl_blocks[0] * instr_w + (cc.lvl_blocks[1] + cc.lvl_blocks[2]) * instr_yz) * dc.wpb
+                            : 0);
     go.g.push_back(G);
   }
 }
@@ -2108,6 +2548,7 @@ static void build_host(Plan *p, const ws_config *cfgs, int n_cfg, const ws_field
     // an item or counting unit takes at most three table entries (a counting unit: its
     // (field, chunk) pair and its item's first unit)
     dsc += 4 * 3 * items;
+    p->own_budget = (int64_t)(3 * items);
   }
   const size_t avail = avail_fn(dsc, total_need);
   size_t scratch = std::min(total_need, avail);
@@ -2226,14 +2667,20 @@ static void build_host(Plan *p, const ws_config *cfgs, int n_cfg, const ws_field
   p->hgrp.reserve(ng);
   p->grp_iv_ok.reserve(ng);
   p->grp_rows_ok.reserve(ng);
+  p->grp_foot_ok.reserve(ng);
+  p->grp_foot_cost.reserve(ng);
   p->grp_slots.reserve(ng);
+  p->grp_blk_slots.reserve(ng);
   p->grp_classes.reserve(ng);
   p->grp_winstr_rows.reserve(ng);
   for (GroupOut &go : gout) {
     p->hgrp.insert(p->hgrp.end(), go.g.begin(), go.g.end());
     p->grp_iv_ok.insert(p->grp_iv_ok.end(), go.iv_ok.begin(), go.iv_ok.end());
     p->grp_rows_ok.insert(p->grp_rows_ok.end(), go.rows_ok.begin(), go.rows_ok.end());
+    p->grp_foot_ok.insert(p->grp_foot_ok.end(), go.foot_ok.begin(), go.foot_ok.end());
+    p->grp_foot_cost.insert(p->grp_foot_cost.end(), go.foot_cost.begin(), go.foot_cost.end());
     p->grp_slots.insert(p->grp_slots.end(), go.slots.begin(), go.slots.end());
+    p->grp_blk_slots.insert(p->grp_blk_slots.end(), go.blk_slots.begin(), go.blk_slots.end());
     p->grp_classes.insert(p->grp_classes.end(), go.cls.begin(), go.cls.end());
     p->grp_winstr_rows.insert(p->grp_winstr_rows.end(), go.winstr.begin(), go.winstr.end());
     p->iv_cap = std::max(p->iv_cap, go.iv_cap);
@@ -2321,10 +2768,10 @@ int ws::plan_create_impl(ws_ctx *ctx, const ws_config *cfgs, int n_cfg, const ws
   }
 
   // device buffers
-  // three work-stealing counters per pass (enumeration, row walk, counting); any tuning
-  // makes at most one pass per
-  // (candidate, field), so size for that (retuning may change the pass count)
-  p->grab_bytes = 24 * (p->hfld.size() + 1);
+  // four work-stealing counters per pass (enumeration, row walk, counting, closed form); any
+  // tuning makes at most one pass per (candidate, field), so size for that (retuning may change
+  // the pass count)
+  p->grab_bytes = 32 * (p->hfld.size() + 1);
   p->counters_bytes = p->grab_bytes + (size_t)n_cfg * N_COUNTERS * 8;
   p->d_cfg = p->take(std::max<size_t>(hcfg.size() * sizeof(DCfg), 256));
   p->d_grp = p->take(std::max<size_t>(p->hgrp.size() * sizeof(DGroup), 256));
@@ -2464,7 +2911,7 @@ extern "C" int ws_plan_profile(ws_plan *p, void *stream, ws_profile *out) {
     out->ms_rank = ms;
     cudaEventElapsedTime(&ms, ev[0], ev[2 + 3 * np]);
     out->ms_total = ms;
-    out->enum_items = p->item_begin_end + p->ritem_begin_end;
+    out->enum_items = p->item_begin_end + p->ritem_begin_end + p->fitem_begin_end;
     out->count_items = p->citem_begin_end;
     out->passes = (int64_t)p->passes.size();
     out->upload_bytes = p->upload_bytes;
@@ -2854,8 +3301,8 @@ extern "C" int ws_plan_dry_run(const ws_config *cfgs, int n_cfg, const ws_field 
   out->groups = (int64_t)p.hgrp.size();
   out->passes = (int64_t)p.passes.size();
   out->enum_items = p.item_begin_end;
-  out->row_items = p.ritem_begin_end;
-  out->count_items = p.citem_begin_end;
+  out->row_items = p.ritem_begin_end + p.fitem_begin_end;
+  out->count_items = p.citems_accounted;
   out->access_entries = (int64_t)h.hacc.size();
   out->interval_entries = (int64_t)h.hiv.size();
   out->descriptor_bytes = (int64_t)h.desc_bytes;
