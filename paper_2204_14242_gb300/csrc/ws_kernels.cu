@@ -2,10 +2,11 @@
 //
 //   enum_kernel   persistent, work-stealing CTAs.  Representative block (Sec. 4.2, 4.3):
 //                 every (warp, access instruction) pair exactly -- per-instruction unique
-//                 sectors (L1 request / write-through volumes), half-warp bank cycles and
-//                 the block bitmaps.  Wave / y / z sets of field groups that cannot take
-//                 the row walk: per modelled warp, as sector intervals of row segments
-//                 (segment walk) or address by address.
+//                 sectors (L1 request / write-through volumes) and half-warp bank cycles,
+//                 once per access code where the block's footprints are made elsewhere
+//                 (AccessCodes), else with the block bitmaps.  Wave / y / z sets of field
+//                 groups that cannot take the row walk: per modelled warp, as sector
+//                 intervals of row segments (segment walk) or address by address.
 //   rows_kernel   wave, y set, z set and block footprints.  In closed form where a field's layout
 //                 allows it (ws_footprint.h; nearly always): counted row by row in registers,
 //                 without bitmaps.  Else as whole grid rows: each merged load run of a row is
@@ -443,6 +444,23 @@ __device__ __noinline__ int64_t row_store_sectors(int64_t A0, int64_t step, int3
   return cnt;
 }
 
+// Accesses of a group whose block is only counted (the row walk or the closed form makes its
+// footprints), taken together by what an instruction's counts depend on: its lanes' addresses
+// modulo a sector and the bank period, a multiple `period` of both, which for accesses of one
+// layout is the place of any one address in the period, and the folded points that need it.
+// The 25-point star has 9 such codes among its 26 accesses, the 84 accesses of a lattice Boltzmann
+// step a handful.  The enumeration is bound by the latency of the warps' instruction chains and of
+// a group's staging; its time (GB300), accesses one by one -> codes: 755 25-point candidates
+// 61 -> 41 us, 755 lattice Boltzmann 173 -> 58, 4,000 mixed 517 -> 245, 40 served 100 -> 31.
+// Groups of at most kFewPairs (class warp, access) pairs keep to the list: the codes' three barriers
+// cost more than they save (one 7-point candidate 12.3 us with the list, 14.7 with codes).
+constexpr int kFewPairs = 64;
+struct AccessCodes {
+  int n;              // codes; 0: this group's accesses are taken one by one
+  uint32_t period;
+  int64_t ref;        // byte offset of the group's first access
+};
+
 // Shared-memory images of one field group, staged by the enumeration and row kernels.
 struct StageSmem {
   DCfg *c;
@@ -465,7 +483,54 @@ struct StageSmem {
   // |ddy| of the last kind}
   int32_t (*idst)[kMaxGroupFields];
   int32_t *cov;
+  AccessCodes *codes;   // enumeration only (else null)
 };
+
+// Makes the codes of the staged group (b32: their counts, loads low and stores high; boff: the list
+// of those that occur) or none; ends with a barrier.
+__device__ __forceinline__ void stage_codes(const EnumArgs &a, const StageSmem &m) {
+  const DGroup &G = *m.g;
+  // one code per place in the period, and per first folded point where the block has threads with
+  // fewer points than the fold; as many as the list of 32-bit offsets has entries
+  const uint32_t period = (uint32_t)max(32, a.banks * a.bank_bytes);
+  const DCfg &c = *m.c;
+  const uint32_t bt = fdiv((uint32_t)c.rep, c.fd_gx), bz = fdiv(bt, c.fd_gy), by = bt - bz * (uint32_t)c.g[1];
+  const bool whole = c.fold_axis == 0 || (c.fold_axis == 1 ? ((int)by + 1) * c.B[1] * c.fold <= c.N[1]
+                                                           : ((int)bz + 1) * c.B[2] * c.fold <= c.N[2]);
+  const uint32_t size = period * (whole ? 1u : (uint32_t)c.fold);
+  if (size > (uint32_t)kMaxFoldedAccesses || m.fk[0].words[0] >= ((int64_t)1 << 22) - 4) {
+    if (threadIdx.x == 0) m.codes->n = 0;
+    __syncthreads();
+    return;
+  }
+  for (uint32_t i = threadIdx.x; i < size; i += blockDim.x) m.b32[i] = 0u;
+  if (threadIdx.x == 0) {
+    m.codes->period = period;
+    m.codes->ref = a.acc[m.fk[0].acc_begin].boff;
+  }
+  __syncthreads();
+  for (int k = 0; k < G.f_count; ++k) {
+    const DField &F = m.fk[k];
+    for (int i = threadIdx.x; i < F.n_load + F.n_store; i += blockDim.x) {
+      const DAcc d = a.acc[F.acc_begin + i];
+      const uint32_t at = ((uint32_t)F.base + (uint32_t)d.boff) & (period - 1u);
+      atomicAdd(m.b32 + at + (whole ? 0u : period * (uint32_t)d.kmin), i < F.n_load ? 1u : 0x10000u);
+    }
+  }
+  __syncthreads();
+  // in ascending order: the CTAs that share the group's items must number the codes alike
+  uint2 *const list = reinterpret_cast<uint2 *>(m.boff);
+  if (threadIdx.x < 32) {
+    int have = 0;
+    for (uint32_t i0 = 0; i0 < size; i0 += 32) {
+      const uint32_t n = m.b32[i0 + threadIdx.x], some = __ballot_sync(FULL, n != 0u);
+      if (n) list[have + __popc(some & ((1u << threadIdx.x) - 1u))] = make_uint2(i0 + threadIdx.x, n);
+      have += __popc(some);
+    }
+    if (threadIdx.x == 0) m.codes->n = have;
+  }
+  __syncthreads();
+}
 
 // Stages group gi (and its candidate when it differs from cur_cfg); ends with a barrier.
 // Returns true when the candidate changed.
@@ -547,6 +612,14 @@ __device__ bool stage_group(const EnumArgs &a, int gi, int cur_cfg, const StageS
     if (kv == 0) m.gwi[lv] = wi;
   }
   __syncthreads();
+  if (m.codes) {
+    if (G.rows && a.bank_shift >= 0 && G.n_rep * G.acc_count > kFewPairs) {
+      stage_codes(a, m);
+      if (m.codes->n) return new_cfg;
+    } else if (threadIdx.x == 0) {
+      m.codes->n = 0;
+    }
+  }
   // merged load runs, offsets relative to each field's bitmap origin (the enumeration kernel
   // uses them only for groups without the row walk)
   const int n_runs = (m.cov != nullptr || !G.rows) ? m.ioff[G.f_count] : 0;
@@ -586,6 +659,74 @@ __device__ bool stage_group(const EnumArgs &a, int gi, int cur_cfg, const StageS
   return new_cfg;
 }
 
+struct BlockCounts {
+  uint32_t lb, req, st, bank, addr, wi;
+};
+
+// Item kk of a group whose accesses come as codes: an instruction is a code with its loads and
+// stores; the items share the (class warp, code) pairs evenly, the warps an item's.  tcs: the
+// block's thread coordinates.
+__device__ __forceinline__ BlockCounts block_codes(const EnumArgs &a, const StageSmem &m, const uint32_t *tcs, int64_t kk) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const DGroup &G = *m.g;
+  const DCfg &c = *m.c;
+  BlockCounts o = {0, 0, 0, 0, 0, 0};
+  const uint2 *const codes = reinterpret_cast<const uint2 *>(m.boff);
+  const uint32_t nc = (uint32_t)m.codes->n, np = (uint32_t)G.n_rep * nc, n0 = (uint32_t)G.n0_items;
+  const uint32_t p0 = (uint32_t)((uint64_t)np * (uint32_t)kk / n0), p1 = (uint32_t)((uint64_t)np * (uint32_t)(kk + 1) / n0);
+  const uint32_t per = (p1 - p0 + nwarps - 1) / nwarps;
+  const uint32_t q0 = min(p0 + warp * per, p1), q1 = min(q0 + per, p1);
+  const DField &F = m.fk[0];
+  const uint32_t period = m.codes->period, pshift = 31u - __clz(period);
+  const uint32_t from = ((uint32_t)F.base + (uint32_t)m.codes->ref) & (period - 1u);
+  const uint32_t bt = fdiv((uint32_t)c.rep, c.fd_gx), bx = (uint32_t)c.rep - bt * (uint32_t)c.g[0];
+  const uint32_t bz = fdiv(bt, c.fd_gy), by = bt - bz * (uint32_t)c.g[1];
+  const int32_t faxis = c.fold_axis, fold = c.fold;
+  uint32_t r = q0 / nc, j = q0 - r * nc, mult = 0, at = 0;
+  int kv = 0;
+  bool fresh = true;
+  for (uint32_t pp = q0; pp < q1; ++pp) {
+    if (fresh) {
+      // a class warp's threads: the place of each one's first address
+      fresh = false;
+      mult = G.rep_mult[r];
+      const uint32_t tid = (uint32_t)G.rep_warp[r] * 32u + lane;
+      const uint32_t tc = tid < (uint32_t)c.T ? tcs[tid] : 0u;
+      const int32_t x = (int32_t)bx * c.B[0] + (int32_t)(tc & 1023u);
+      int32_t y = (int32_t)by * c.B[1] + (int32_t)((tc >> 10) & 1023u);
+      int32_t z = (int32_t)bz * c.B[2] + (int32_t)(tc >> 20);
+      if (faxis == 1) y *= fold;
+      if (faxis == 2) z *= fold;
+      kv = 0;
+      if (tid < (uint32_t)c.T && x < c.N[0] && y < c.N[1] && z < c.N[2])
+        kv = faxis == 1 ? min(fold, c.N[1] - y) : faxis == 2 ? min(fold, c.N[2] - z) : 1;
+      if (j == 0u) {
+        if (G.first_of_cfg) o.lb += mult * __reduce_add_sync(FULL, (uint32_t)kv);
+        o.addr += mult * __reduce_add_sync(FULL, (uint32_t)m.gad[0][kv]);
+        o.wi += mult * (uint32_t)m.gwi[0];
+      }
+      const int64_t lin = F.stride[0] * x + F.stride[1] * y + F.stride[2] * z;
+      const int64_t r0 = F.base + (int64_t)F.esize * lin - 32 * F.lo[0] + m.codes->ref;
+      if (r0 < 0 || r0 >= F.words[0] << 10) kv = 0;
+      at = (uint32_t)r0 - from + period;   // (a period is added, so that none falls below the origin)
+    }
+    const uint2 cd = codes[j];
+    const uint32_t rel = at + (cd.x & (period - 1u)), nl = cd.y & 0xffffu, ns = cd.y >> 16;
+    const bool act = (int)(cd.x >> pshift) < kv;
+    const uint32_t nsec = mult * warp_distinct_sectors(rel, act);
+    o.req += nsec * nl;
+    o.st += nsec * ns;
+    o.bank += mult * (nl + ns) * (uint32_t)bank_cycles_rel32(rel, act, lane, (uint32_t)a.bank_shift,
+                                                               (uint32_t)(a.banks - 1), (uint32_t)a.pair_dist);
+    if (++j == nc) {
+      j = 0;
+      ++r;
+      fresh = true;
+    }
+  }
+  return o;
+}
+
 __global__ void __launch_bounds__(512, 2) enum_kernel(EnumArgs a) {
   __shared__ DCfg s_c;
   __shared__ DGroup s_g;
@@ -606,6 +747,7 @@ __global__ void __launch_bounds__(512, 2) enum_kernel(EnumArgs a) {
   __shared__ int32_t s_gad[2][17];                     // group's issued accesses per thread with kv points
   __shared__ int32_t s_gwi[2];                         // group's access instructions ([0] levels 0-1, [1] 2-3)
   __shared__ long long s_item;
+  __shared__ AccessCodes s_codes;
   // merged load intervals of an interval-walk group (dynamic): offset, extent, field
   extern __shared__ __align__(16) unsigned char s_dyn[];
   const int iv_cap16 = (a.iv_cap + 15) & ~15;
@@ -613,7 +755,7 @@ __global__ void __launch_bounds__(512, 2) enum_kernel(EnumArgs a) {
   uint32_t *const s_iext = reinterpret_cast<uint32_t *>(s_dyn + 8 * iv_cap16);
   uint8_t *const s_iaf = s_dyn + 12 * iv_cap16;
   const StageSmem sm{&s_c, &s_g, s_fk, s_loff, s_soff, s_ioff, s_af, s_boff, s_b32, s_kmin, s_gad, s_gwi,
-                     s_ibo, s_iext, s_iaf, nullptr, nullptr};
+                     s_ibo, s_iext, s_iaf, nullptr, nullptr, &s_codes};
 
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t warp = threadIdx.x >> 5;
@@ -659,7 +801,15 @@ __global__ void __launch_bounds__(512, 2) enum_kernel(EnumArgs a) {
     uint32_t acc_lb = 0, acc_lw = 0, acc_req = 0, acc_st = 0, acc_bank = 0, acc_sreq = 0, acc_addr = 0, acc_wi = 0;
     uint32_t bad = 0;
 
-    if (blk) {
+    if (blk && s_codes.n) {
+      const BlockCounts o = block_codes(a, sm, s_tc, kk);
+      acc_lb = o.lb;
+      acc_req = o.req;
+      acc_st = o.st;
+      acc_bank = o.bank;
+      acc_addr = o.addr;
+      acc_wi = o.wi;
+    } else if (blk) {
       // ---- representative block (Sec. 4.2, 4.3): every (warp, instruction) exactly --
       // distinct sectors per instruction (L1 requests / write-through stores), the block
       // footprint bitmaps, and half-warp bank cycles.  Each warp takes a contiguous run of
@@ -1951,7 +2101,7 @@ __global__ void __launch_bounds__(256, 2) rows_kernel(EnumArgs a) {
   uint32_t *const s_iext = reinterpret_cast<uint32_t *>(s_dyn + 8 * iv_cap16);
   uint8_t *const s_iaf = s_dyn + 12 * iv_cap16;
   const StageSmem sm{&s_c, &s_g, s_fk, s_loff, s_soff, s_ioff, s_af, s_boff, nullptr, s_kmin, s_gad, s_gwi,
-                     s_ibo, s_iext, s_iaf, s_idst, s_cov};
+                     s_ibo, s_iext, s_iaf, s_idst, s_cov, nullptr};
 
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t warp = threadIdx.x >> 5;
