@@ -51,6 +51,7 @@ struct ModelArgs {
   const int64_t *counters;
   ws_result *results;
   double *keys;                    // rank keys (t_pred rounded to 40 bits)
+  int32_t *rank;                   // set to 0 for the ranking that follows
   int32_t n;
   DHw hw;
 };
@@ -68,7 +69,7 @@ cudaError_t launch_rows(const EnumArgs &args, int grid, cudaStream_t st);
 cudaError_t launch_count(const CountArgs &args, int grid, cudaStream_t st);
 cudaError_t launch_model(const ModelArgs &args, cudaStream_t st);
 cudaError_t launch_rank(const RankArgs &args, cudaStream_t st);
-cudaError_t launch_keys(const ws_result *res, int n, double *keys, cudaStream_t st);
+cudaError_t launch_keys(const ws_result *res, int n, double *keys, int32_t *rank, cudaStream_t st);
 cudaError_t enum_occupancy(int threads, int iv_cap, int *blocks_per_sm);
 size_t enum_dyn_smem(int iv_cap);
 cudaError_t rows_occupancy(int iv_cap, int *blocks_per_sm);

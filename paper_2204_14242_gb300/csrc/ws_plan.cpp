@@ -1860,6 +1860,7 @@ int ws_plan::enqueue(cudaStream_t st, std::vector<cudaEvent_t> *ev, ws_profile *
   ma.counters = (const int64_t *)((char *)dev(d_counters) + grab_bytes);
   ma.results = (ws_result *)dev(d_results);
   ma.keys = (double *)dev(d_keys);
+  ma.rank = (int32_t *)dev(d_rank);
   ma.n = n_cfg;
   ma.hw = dhw;
   CU(launch_model(ma, st));
@@ -1970,6 +1971,7 @@ int ws_plan::run_plain_launches(cudaStream_t st) {
     ma.counters = counters + (int64_t)i * N_COUNTERS;
     ma.results = (ws_result *)dev(d_results) + i;
     ma.keys = (double *)dev(d_keys) + i;
+    ma.rank = (int32_t *)dev(d_rank) + i;
     ma.n = 1;
     ma.hw = dhw;
     CU(launch_model(ma, st));
@@ -3129,7 +3131,7 @@ static int estimate_pipelined(ws_ctx *ctx, const ws_config *cfgs, int n_cfg, con
     if (e == cudaSuccess) e = ej3;
   }
   if (rc == WS_OK && e == cudaSuccess) {
-    e = launch_keys((const ws_result *)(b + o_res), n_cfg, (double *)(b + o_keys), st);
+    e = launch_keys((const ws_result *)(b + o_res), n_cfg, (double *)(b + o_keys), (int32_t *)(b + o_rnk), st);
     if (e == cudaSuccess) {
       RankArgs ra;
       ra.keys = (const double *)(b + o_keys);
@@ -3333,7 +3335,8 @@ extern "C" int ws_rank(ws_ctx *ctx, const ws_result *res, int n, int32_t *order_
     int32_t seg[2] = {0, n};
     cudaError_t e = cudaMemcpyAsync(b + o_res, res, rb, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b + o_seg, seg, sizeof(seg), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_keys((const ws_result *)(b + o_res), n, (double *)(b + o_keys), st);
+    if (e == cudaSuccess)
+      e = launch_keys((const ws_result *)(b + o_res), n, (double *)(b + o_keys), (int32_t *)(b + o_rnk), st);
     if (e == cudaSuccess) {
       RankArgs ra;
       ra.keys = (const double *)(b + o_keys);
