@@ -1,7 +1,7 @@
 // Closed-form footprints: unique sectors, unique lines and overlaps of the representative
-// block, the wave and the y / z sets of a field, counted row by row without a bitmap.  The
-// geometry here is shared by the row-walk kernel (ws_kernels.cu) and by the host check of
-// the same rule (ws_plan.cpp).
+// block, the wave and the y / z sets of a field, counted row by row without a bitmap: the
+// geometry and the counting of a row, used by rows_kernel (ws_kernels.cu).  Which fields take
+// it is decided by closed_form_ok (ws_plan.cpp).
 //
 // The points a level updates, whatever the folding, are the valid points of its blocks; the
 // level's load (store) footprint is those points plus the raw offsets.  A level is a
