@@ -14,7 +14,8 @@
 //   class S: runs that start at the level's first block of its first block row,
 // and within a class the ranges overlap or touch whenever a run is at least as long as the
 // offsets are spread (checked by the host, closed_form_ok): the class is one byte range.
-// Addresses matter modulo a line only, so neither the level's size nor its position is limited.
+// Addresses matter modulo a line only, so the level's position is not limited; its size is only
+// by the 32-bit counts of FootCounts (fewer than 2^32 sectors, checked by the host likewise).
 // Two neighbouring target rows may still share sectors (row ends off the sector grid, offsets
 // reaching over the row's end), so sectors and lines are counted in cells: the cell of target
 // row t holds the lines from floor((A(t) + hmin) / 128) up to the next row's, A(t) being the
@@ -295,7 +296,9 @@ WS_HD bool foot_key(const FootGeo &g, int32_t r, int32_t n, int32_t key[4]) {
 }
 
 // What a task counts: sectors and lines of the first level, lines of the y and z sets, the
-// first level's sectors shared with the y set, and with the z set outside the y set.
+// first level's sectors shared with the y set, and with the z set outside the y set.  A level has
+// fewer than 2^32 sectors (closed_form_ok), so no lane's and no warp's sum overflows; ovz is
+// added to and taken from modulo 2^32.
 struct FootCounts {
   uint32_t sec, lin, ylin, zlin, ovy, ovz;
 };

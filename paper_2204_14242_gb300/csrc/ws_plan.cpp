@@ -665,11 +665,16 @@ struct RowsPerPlane {
 //  * a row's ranges, from the lowest byte any starts at to the highest any ends at, leave a line
 //    to spare in two pitches, so that they reach no further than the next row's cell;
 //  * within a level's class of runs the ranges overlap or touch: the offsets' rests are spread by
-//    at most the shortest run and one sector.
+//    at most the shortest run and one sector;
+//  * the wave holds fewer than 2^32 sectors: the counts of an item are 32-bit sums.  At most that
+//    many are the sectors of the address range, and the accesses its threads issue (touched: one
+//    sector each; the y and z sets are parts of the wave moved).  64-bit sums need no such limit,
+//    but take 4,000 mixed candidates 1.94 -> 2.17 ms (GB300), and a wave that reaches it reads
+//    128 GiB of one array; such a field is left to the address walk.
 template <class Run>
 static void closed_form_ok(const ws_field &F, const FieldFold &ff, int mask, const int64_t pb_lo[2][3],
-                           const int64_t pb_hi[2][3], int64_t n0, int64_t run_any, Run shortest_run,
-                           RowsPerPlane &rows, DField &df) {
+                           const int64_t pb_hi[2][3], int64_t n0, int64_t touched, int64_t run_any,
+                           Run shortest_run, RowsPerPlane &rows, DField &df) {
   const int64_t P = (int64_t)F.elem_bytes * F.stride[1], esx = (int64_t)F.elem_bytes * F.stride[0];
   if (esx < 0 || esx > 32) return;
   const int64_t spread = std::max(ff.dsp_spread[0], ff.dsp_spread[1]);
@@ -706,6 +711,7 @@ static void closed_form_ok(const ws_field &F, const FieldFold &ff, int mask, con
     if (!(mask & (1 << lv))) continue;
     if (spread > esx * (run_any - 1) + 32 && spread > esx * (shortest_run(lv) - 1) + 32) continue;
     if (lv == 0 && df.words[0] >= ((int64_t)1 << 22)) continue;   // (the block's per-instruction counts)
+    if (lv == 1 && std::min(32 * df.words[1], touched) >= ((int64_t)1 << 32)) continue;
     df.closed |= lv == 0 ? 2 : 1;
   }
 }
@@ -1202,7 +1208,10 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     df.n_dsp_s = (int16_t)ff->n_dsp[1];
     df.closed = 0;
     df.q = 1;
-    if (ff->dsp_ok) closed_form_ok(F, *ff, mask, pb_lo, pb_hi, c.N[0], run_any, shortest_run, plane_rows, df);
+    if (ff->dsp_ok) {
+      const int64_t touched = weff * T * std::max(df.n_load, df.n_store);
+      closed_form_ok(F, *ff, mask, pb_lo, pb_hi, c.N[0], touched, run_any, shortest_run, plane_rows, df);
+    }
     for (int kv = 0; kv <= 16; ++kv) {
       df.cnt_load[kv] = ff->cnt_load[kv];
       df.cnt_store[kv] = ff->cnt_store[kv];
