@@ -112,17 +112,17 @@ struct DField {
   uint8_t zmove;          // closed form: the z set is the wave moved by whole planes, by zmove - 1 bytes modulo 128
                           //   (0: it is not)
   int32_t q;              // closed form: rows from plane to plane
-  uint32_t fq_m, fq_s;    //   and its FastDiv
+  uint32_t fq_m;          //   and its FastDiv (with fq_s)
   int16_t n_dsp_l, n_dsp_s;   // closed form: displacements of the loads / of the stores (behind the intervals)
   int32_t y_span_l, y_span_s; //   largest less smallest displacement within a plane (>= q: unknown)
   uint8_t mult_l, mult_s;     //   fields of the group whose loads / stores this one's stand for (0: another one's do)
-  uint8_t pad8b[2];
+  uint8_t fq_s;
+  uint8_t zshift;         // 1: the z set's sectors are the wave's moved by whole lines (loads)
   int32_t n_iv_unc;       // merged load intervals without a covering run (they come first)
   int32_t n_iv_zc;        // those covered from another z row (they come next; the rest last)
   int16_t cov_dy, cov_dz; // largest |row displacement| from an interval to its covering run
   int16_t cov_dy_y;       // largest |ddy| of the intervals covered within their z row
   int16_t pad16;
-  int32_t zshift;         // 1: the z set's sectors are the wave's moved by whole lines (loads)
   int32_t zc_lo, zc_hi;   // zshift: sectors (from the wave origin) bounding the wave's addresses
   int16_t cnt_load[17];   // folded loads issued by a thread with kv valid points
   int16_t cnt_store[17];  // folded stores likewise

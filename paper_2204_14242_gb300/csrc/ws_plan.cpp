@@ -17,6 +17,7 @@
 #include <memory>
 #include <memory_resource>
 #include <unordered_map>
+#include <unordered_set>
 #include <mutex>
 #include <new>
 #include <set>
@@ -704,7 +705,7 @@ static void closed_form_ok(const ws_field &F, const FieldFold &ff, int mask, con
   df.q = (int32_t)q;
   if (rows.fq.d != (uint32_t)q) rows.fq = make_fastdiv((uint32_t)q);
   df.fq_m = rows.fq.m;
-  df.fq_s = rows.fq.s;
+  df.fq_s = (uint8_t)rows.fq.s;
   df.y_span_l = (int32_t)(planes ? std::min(ff.dsp_y[0], q) : q);
   df.y_span_s = (int32_t)(planes ? std::min(ff.dsp_y[1], q) : q);
   for (int lv = 0; lv < 2; ++lv) {
@@ -2284,8 +2285,7 @@ static void compile_all(const ws_config *cfgs, int n_cfg, const ws_field *fld, i
         const size_t cr = 256;   // the smallest row-walk item
         for (size_t k = 0; k < cc.f.size(); ++k) {
           const int64_t nacc = cc.acc_off[k + 1] - cc.acc_off[k], niv = cc.iv_off[k + 1] - cc.iv_off[k];
-          // the displacements of the closed form are left to the estimate's slack (a group per
-          // field, owner-table entries of items the closed form does not make) and headroom
+          // (the displacements of the closed form: see descriptor_extra)
           cc.dsc_bytes += sizeof(DField) + sizeof(DGroup) + (size_t)nacc * sizeof(DAcc) +
                           (size_t)cc.f[k].n_iv * sizeof(DIv);
           cc.need_sum += (size_t)cc.need_words[k] * 4;
@@ -2317,7 +2317,7 @@ int ws::plan_requirements(const ws_config *cfgs, int n_cfg, const ws_field *fld,
     if (compile_config(cfgs[i], fld, n_fld, acc, n_acc, *hw, cc, &cache) != WS_OK) continue;
     for (size_t k = 0; k < cc.f.size(); ++k) {
       dsc += sizeof(DField) + sizeof(DGroup) + (size_t)(cc.acc_off[k + 1] - cc.acc_off[k]) * sizeof(DAcc) +
-             (size_t)cc.f[k].n_iv * sizeof(DIv);
+             (size_t)(cc.iv_off[k + 1] - cc.iv_off[k]) * sizeof(DIv);
       scr += (size_t)cc.need_words[k] * 4;
       mf = std::max(mf, (size_t)cc.need_words[k] * 4);
     }
@@ -2328,6 +2328,9 @@ int ws::plan_requirements(const ws_config *cfgs, int n_cfg, const ws_field *fld,
   *scratch_bytes = scr;
   return WS_OK;
 }
+
+// Four work-stealing counters per pass (enumeration, row walk, counting, closed form).
+constexpr size_t kGrabBytes = 4 * sizeof(unsigned long long);
 
 // Host half of plan creation: compiles the candidates, deduplicates their access lists,
 // builds field groups and cuts passes.  avail_fn(descriptor bytes, bitmap bytes of all
@@ -2527,6 +2530,34 @@ static void build_groups(Plan *p, int i, const Compiled &cc, const ws_hw &hw, Gr
   }
 }
 
+// Room that plan creation leaves in the arena beside the descriptor estimate.
+constexpr size_t kDescHeadroom = (size_t)8 << 20;
+
+// Bytes that the descriptor estimate does not list, less the headroom that holds them in an
+// ordinary batch: the work-stealing counters of the passes (at most one a field), and the
+// closed form's displacements, which grow with the accesses (1,500 fields of 961 loads in rows of
+// their own have 23 MB).  Only what the headroom cannot hold is added, so that a batch that fits a
+// given arena without them still does.
+static size_t descriptor_extra(const CompileArena &ca, const std::vector<int> &status) {
+  const size_t room = kDescHeadroom - ((size_t)256 << 10);   // (the rest: granularity of the buffers)
+  std::unordered_set<uint64_t> seen;
+  size_t bytes = 0;
+  for (int once = 0; once < 2; ++once) {   // every field's list, then (seldom) shared ones once
+    bytes = 0;
+    for (size_t i = 0; i < status.size(); ++i) {
+      if (status[i] != WS_OK) continue;
+      const Compiled &cc = *ca.comp[i];
+      for (size_t k = 0; k < cc.f.size(); ++k) {
+        bytes += kGrabBytes;
+        if (!once || cc.fkey[k] == kNoShare || seen.insert(cc.fkey[k]).second)
+          bytes += (size_t)(cc.f[k].n_dsp_l + cc.f[k].n_dsp_s) * sizeof(DDsp);
+      }
+    }
+    if (bytes <= room) return 0;
+  }
+  return bytes - room;
+}
+
 static void build_host(Plan *p, const ws_config *cfgs, int n_cfg, const ws_field *fld, int n_fld,
                        const ws_access *acc, int n_acc, const ws_hw *hw,
                        const std::function<size_t(size_t, size_t)> &avail_fn, HostDesc &h) {
@@ -2561,6 +2592,7 @@ static void build_host(Plan *p, const ws_config *cfgs, int n_cfg, const ws_field
     dsc += 4 * 3 * items;
     p->own_budget = (int64_t)(3 * items);
   }
+  dsc += descriptor_extra(ca, status);
   const size_t avail = avail_fn(dsc, total_need);
   size_t scratch = std::min(total_need, avail);
   scratch = std::max<size_t>(scratch, 16);
@@ -2741,7 +2773,7 @@ int ws::plan_create_impl(ws_ctx *ctx, const ws_config *cfgs, int n_cfg, const ws
         ctx->oneshot_off = -1;
         ctx->oneshot_bytes = 0;
         size_t room = ctx->arena->largest_free();
-        room = room > dsc + (8 << 20) ? room - dsc - (8 << 20) : 0;
+        room = room > dsc + kDescHeadroom ? room - dsc - kDescHeadroom : 0;
         const size_t want = std::min((need + 255) & ~(size_t)255, room & ~(size_t)255);   // whole bitmaps: one pass
         const int64_t o = want >= 256 ? ctx->arena->alloc(want) : -1;
         if (o >= 0) {
@@ -2756,7 +2788,7 @@ int ws::plan_create_impl(ws_ctx *ctx, const ws_config *cfgs, int n_cfg, const ws
       }
     }
     size_t avail = ctx->arena->largest_free();
-    avail = avail > dsc + (8 << 20) ? avail - dsc - (8 << 20) : 0;
+    avail = avail > dsc + kDescHeadroom ? avail - dsc - kDescHeadroom : 0;
     if (ext_scratch >= 0) avail = ext_scratch_bytes;
     if (scratch_cap) avail = std::min(avail, scratch_cap);
     return avail;
@@ -2779,10 +2811,9 @@ int ws::plan_create_impl(ws_ctx *ctx, const ws_config *cfgs, int n_cfg, const ws
   }
 
   // device buffers
-  // four work-stealing counters per pass (enumeration, row walk, counting, closed form); any
-  // tuning makes at most one pass per (candidate, field), so size for that (retuning may change
-  // the pass count)
-  p->grab_bytes = 32 * (p->hfld.size() + 1);
+  // any tuning makes at most one pass per (candidate, field), so size for that (retuning may
+  // change the pass count)
+  p->grab_bytes = kGrabBytes * (p->hfld.size() + 1);
   p->counters_bytes = p->grab_bytes + (size_t)n_cfg * N_COUNTERS * 8;
   p->d_cfg = p->take(std::max<size_t>(hcfg.size() * sizeof(DCfg), 256));
   p->d_grp = p->take(std::max<size_t>(p->hgrp.size() * sizeof(DGroup), 256));
@@ -3186,7 +3217,7 @@ static int estimate_pipelined(ws_ctx *ctx, const ws_config *cfgs, int n_cfg, con
     for (int i : short_of_room) {
       size_t dsc = 0, scr = 0, mf = 0;
       plan_requirements(cfgs + i, 1, fld, n_fld, acc, n_acc, hw, &dsc, &scr, &mf);
-      if (mf + ((size_t)8 << 20) <= room) return WS_ENOMEM;
+      if (mf + kDescHeadroom <= room) return WS_ENOMEM;
     }
   }
   return rc;
