@@ -14,6 +14,7 @@
 #include "ws_internal.h"
 
 namespace ws {
+struct EnumArgs;
 
 // First-fit allocator over one device buffer; offsets are 256-byte aligned.
 struct Arena {
@@ -195,6 +196,7 @@ struct ws_plan {
   int upload_fields(cudaStream_t st);
   int grid_for(int threads, int64_t items, bool counting) const;
   int grid_rows(int64_t items, int64_t fitems) const;
+  int enqueue_rows(const ws::EnumArgs &args, bool apart, cudaStream_t st, int *launches);
   int bank_shift() const;
   int enqueue(cudaStream_t st, std::vector<cudaEvent_t> *ev, ws_profile *prof);
   // Recorded after the descriptor uploads: launches on any stream wait for it (a graph

@@ -221,6 +221,7 @@ struct DPass {
   int64_t citem_lo, citem_hi;  // counting items of the pass
   int32_t cf_lo, cf_hi;        // (candidate, field) index range
   int32_t grp_lo, grp_hi;      // field-group index range
+  bool apart;                  // a launch for the row-walk items and one for the closed-form items
   int64_t words;               // scratch words [0, words) holding the pass's bitmaps
 };
 

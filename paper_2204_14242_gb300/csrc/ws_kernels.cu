@@ -407,8 +407,8 @@ __device__ __forceinline__ int64_t sum_floor32(int64_t n, int64_t P, int64_t c) 
 // Segments repeat from block to block with the address step B0 * step, so each segment
 // position contributes two floor sums over the row's whole blocks; the block cut by N0
 // is counted directly.  A0 + step * x is the relative address of point x of the row.
-__device__ __noinline__ int64_t row_store_sectors(int64_t A0, int64_t step, int32_t B0, int32_t N0, int32_t full_end,
-                                     uint32_t t, uint32_t bxa, uint32_t bxb) {
+__device__ __forceinline__ int64_t row_store_sectors(int64_t A0, int64_t step, int32_t B0, int32_t N0, int32_t full_end,
+                                                     uint32_t t, uint32_t bxa, uint32_t bxb) {
   auto direct = [&](int64_t x0, int64_t x1) -> int64_t {
     const int64_t p = A0 + step * x0, q = A0 + step * x1;
     return (max(p, q) >> 5) - (min(p, q) >> 5) + 1;
@@ -442,6 +442,12 @@ __device__ __noinline__ int64_t row_store_sectors(int64_t A0, int64_t step, int3
     ta = tb;
   }
   return cnt;
+}
+
+// The same out of line, for the closed form's kernel, whose code has to stay short.
+__device__ __noinline__ int64_t row_store_sectors_call(int64_t A0, int64_t step, int32_t B0, int32_t N0, int32_t full_end,
+                                                       uint32_t t, uint32_t bxa, uint32_t bxb) {
+  return row_store_sectors(A0, step, B0, N0, full_end, t, bxa, bxb);
 }
 
 // Accesses of a group whose block is only counted (the row walk or the closed form makes its
@@ -1914,7 +1920,7 @@ __device__ __noinline__ void foot_stats(const EnumArgs &a, const DGroup &G, unsi
           const unsigned long long hit = cache[at];
           uint32_t val = (uint32_t)hit;
           if ((uint32_t)(hit >> 32) != tag) {
-            val = (uint32_t)row_store_sectors((int64_t)A0, sxe, c.B[0], c.N[0], c.full_end, t, bxa, bxb);
+            val = (uint32_t)row_store_sectors_call((int64_t)A0, sxe, c.B[0], c.N[0], c.full_end, t, bxa, bxb);
             cache[at] = ((unsigned long long)tag << 32) | val;
           }
           sum += (unsigned long long)val * ct;
@@ -2067,8 +2073,11 @@ __device__ __forceinline__ void foot_items(const EnumArgs &a, FootSmem &m) {
 // red.or and 0.092 ms of counting 179 MB of bitmaps -> 0.230 and 0.018 ms; 755 lattice Boltzmann
 // candidates: 1.163 and 0.984 -> 0.252 and 0.002 ms (3.66 GB of bitmaps not read, fields that are
 // whole-line copies counted once); 4,000 mixed candidates: 2.66 and 1.32 -> 1.90 and 0.06 ms.
-__global__ void __launch_bounds__(256, 2) rows_kernel(EnumArgs a) {
-
+// Without closed-form items the row walk has an instance of its own, 64 registers and four CTAs an
+// SM: 755 25-point candidates with descending rows 0.287 -> 0.196 ms, 755 lattice Boltzmann ones whose
+// planes are no whole number of rows apart 1.84 -> 1.46 ms.
+template <bool kFoot>
+__global__ void __launch_bounds__(256, kFoot ? 2 : 4) rows_kernel(EnumArgs a) {
   __shared__ DCfg s_c;
   __shared__ DGroup s_g;
   __shared__ DField s_fk[kMaxGroupFields];
@@ -2350,8 +2359,12 @@ __global__ void __launch_bounds__(256, 2) rows_kernel(EnumArgs a) {
                                              ((unsigned long long)((r.t * (uint32_t)s_c.B[0]) & 31u) << 5) |
                                              ((unsigned long long)r.bxa << 10) | ((unsigned long long)r.bxb << 37);
               if (s_memo_key[threadIdx.x] != key) {
-                s_memo_val[threadIdx.x] =
-                    (uint32_t)row_store_sectors(A0, sxe, s_c.B[0], s_c.N[0], s_c.full_end, r.t, r.bxa, r.bxb);
+                if constexpr (kFoot)
+                  s_memo_val[threadIdx.x] =
+                      (uint32_t)row_store_sectors_call(A0, sxe, s_c.B[0], s_c.N[0], s_c.full_end, r.t, r.bxa, r.bxb);
+                else
+                  s_memo_val[threadIdx.x] =
+                      (uint32_t)row_store_sectors(A0, sxe, s_c.B[0], s_c.N[0], s_c.full_end, r.t, r.bxa, r.bxb);
                 s_memo_key[threadIdx.x] = key;
               }
               sreq += s_memo_val[threadIdx.x];
@@ -2390,7 +2403,7 @@ __global__ void __launch_bounds__(256, 2) rows_kernel(EnumArgs a) {
   // then the closed-form items, a warp each, their state in the room of the row walk's access
   // offsets (every warp has passed the last item's barriers)
   static_assert(sizeof(FootSmem) * (kRowsThreads / 32) <= sizeof(s_boff) && alignof(FootSmem) <= 16, "FootSmem in s_boff");
-  foot_items(a, reinterpret_cast<FootSmem *>(s_boff)[threadIdx.x >> 5]);
+  if constexpr (kFoot) foot_items(a, reinterpret_cast<FootSmem *>(s_boff)[threadIdx.x >> 5]);
 }
 
 __constant__ int kCountDst[12] = {C_BLK_LS, C_BLK_LL, C_BLK_SS, C_BLK_SL, C_W_LS, C_W_LL,
@@ -2814,7 +2827,8 @@ static cudaError_t enum_allow_smem(size_t dyn) {
   std::lock_guard<std::mutex> g(mu);
   if (dyn <= allowed[dev]) return cudaSuccess;
   e = cudaFuncSetAttribute(enum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  for (auto *rows : {rows_kernel<false>, rows_kernel<true>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
   if (e == cudaSuccess) allowed[dev] = dyn;
   return e;
 }
@@ -2830,7 +2844,8 @@ cudaError_t launch_rows(const EnumArgs &args, int grid, cudaStream_t st) {
   const size_t dyn = enum_dyn_smem(args.iv_cap);
   cudaError_t e = enum_allow_smem(dyn);
   if (e != cudaSuccess) return e;
-  rows_kernel<<<grid, kRowsThreads, dyn, st>>>(args);
+  if (args.fitem_hi > args.fitem_lo) rows_kernel<true><<<grid, kRowsThreads, dyn, st>>>(args);
+  else rows_kernel<false><<<grid, kRowsThreads, dyn, st>>>(args);
   return cudaGetLastError();
 }
 cudaError_t launch_count(const CountArgs &args, int grid, cudaStream_t st) {
@@ -2862,11 +2877,12 @@ cudaError_t enum_occupancy(int threads, int iv_cap, int *blocks_per_sm) {
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, enum_kernel, threads, dyn);
 }
-cudaError_t rows_occupancy(int iv_cap, int *blocks_per_sm) {
+cudaError_t rows_occupancy(int iv_cap, bool foot, int *blocks_per_sm) {
   const size_t dyn = enum_dyn_smem(iv_cap);
   cudaError_t e = enum_allow_smem(dyn);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, rows_kernel, kRowsThreads, dyn);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, foot ? rows_kernel<true> : rows_kernel<false>,
+                                                       kRowsThreads, dyn);
 }
 cudaError_t count_occupancy(int *blocks_per_sm) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, count_kernel, kCountThreads, 0);

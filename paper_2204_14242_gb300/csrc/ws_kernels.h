@@ -72,7 +72,7 @@ cudaError_t launch_rank(const RankArgs &args, cudaStream_t st);
 cudaError_t launch_keys(const ws_result *res, int n, double *keys, int32_t *rank, cudaStream_t st);
 cudaError_t enum_occupancy(int threads, int iv_cap, int *blocks_per_sm);
 size_t enum_dyn_smem(int iv_cap);
-cudaError_t rows_occupancy(int iv_cap, int *blocks_per_sm);
+cudaError_t rows_occupancy(int iv_cap, bool foot, int *blocks_per_sm);   // foot: with closed-form items
 constexpr int kRowsThreads = 256;
 constexpr int kCountThreads = 256;   // counting kernel: threads per CTA
 constexpr int kCountMaxWords = 65536;   // most bitmap words of one counting unit of a field without page flags

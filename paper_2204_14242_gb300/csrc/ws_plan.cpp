@@ -1426,6 +1426,15 @@ static void default_tuning(ws_tuning &t) {
   if (t.walk != WS_WALK_ADDRESS && t.walk != WS_WALK_SEGMENT) t.walk = WS_WALK_INTERVAL;
 }
 
+// A pass whose row-walk items outweigh its closed-form ones has a launch for each kind, as the row
+// walk alone runs with four CTAs an SM and together with the closed form with two: work of the row
+// walk (slots times the group's runs and stores, some 7 ns a thousand of them) of at least
+// kApartWork, and kApartRatio times the closed form's estimate (some 1.1 ns a thousand instructions).
+// 755 25-point candidates of which 75 / 95 % have descending rows: together 444 / 453 us a step, apart
+// 415 / 395; 50 % (below the ratio) 408 and 406; 90 of 100 (below the work) 150 and 178 (GB300).
+static constexpr int64_t kApartWork = 14000000;
+static constexpr double kApartRatio = 0.35;
+
 // Closed-form items are shares of a field of foot_unit estimated warp instructions (ClosedFormCost),
 // at most kFootParts of them: three for every resident warp, or two while those stay below
 // kFootUnitSmall (an item's set-up, some 20 us with the instructions' fetch, then costs more than
@@ -1546,17 +1555,23 @@ void ws_plan::layout() {
   {
     DPass cur;
     memset(&cur, 0, sizeof(cur));
+    int64_t walk_work = 0, foot_work = 0;   // of the pass
     int64_t used = 0;
+    auto close_pass = [&](int g_end, int cf_end) {
+      cur.cf_hi = cf_end;
+      cur.grp_hi = g_end;
+      cur.item_hi = items;
+      cur.ritem_hi = ritems;
+      cur.fitem_hi = fitems;
+      cur.words = used;
+      cur.apart = foot_work > 0 && walk_work >= kApartWork && (double)walk_work >= kApartRatio * (double)foot_work;
+      walk_work = foot_work = 0;
+      passes.push_back(cur);
+    };
     for (int g = 0; g < ng; ++g) {
       DGroup &G = hgrp[(size_t)g];
       if (used + gneed[(size_t)g] > cap && g > cur.grp_lo) {
-        cur.cf_hi = G.f_begin;
-        cur.grp_hi = g;
-        cur.item_hi = items;
-        cur.ritem_hi = ritems;
-        cur.fitem_hi = fitems;
-        cur.words = used;
-        passes.push_back(cur);
+        close_pass(g, G.f_begin);
         memset(&cur, 0, sizeof(cur));
         cur.item_lo = items;
         cur.ritem_lo = ritems;
@@ -1576,16 +1591,12 @@ void ws_plan::layout() {
       G.fitem_begin = fitems;
       G.f_parts = G.foot ? (int32_t)std::max<int64_t>(1, std::min<int64_t>(kFootParts, grp_foot_cost[(size_t)g] / foot_unit)) : 0;
       fitems += (int64_t)__builtin_popcount(G.foot_fields) * G.f_parts;
+      walk_work += row_slots(g) * (G.n_iv + G.n_stores);
+      if (G.foot) foot_work += grp_foot_cost[(size_t)g] * __builtin_popcount(G.foot_fields);
       if (G.rows) ritems += ceil_div(row_slots(g), chunk_rows());
       else if (G.levels & 2) items += ceil_div(G.mw_end - G.mw_block, tune.chunk_warps);
     }
-    cur.cf_hi = (int)hfld.size();
-    cur.grp_hi = ng;
-    cur.item_hi = items;
-    cur.ritem_hi = ritems;
-    cur.fitem_hi = fitems;
-    cur.words = used;
-    if (ng > 0) passes.push_back(cur);
+    if (ng > 0) close_pass(ng, (int)hfld.size());
   }
   // the warps take the closed-form items in order: those of the longest parts first (by powers of
   // two), so that none of them is left for the end
@@ -1770,16 +1781,37 @@ int ws_plan::bank_shift() const {
   return sh;
 }
 
-// CTAs of the row-walk kernel: one per row-walk item, one per eight warps' closed-form items.
+// CTAs of rows_kernel (of its instance without closed-form items where there are none): one per
+// row-walk item, one per eight warps' closed-form items.
 int ws_plan::grid_rows(int64_t items, int64_t fitems) const {
   int occ = 1;
-  rows_occupancy(iv_cap, &occ);
+  rows_occupancy(iv_cap, fitems > 0, &occ);
   if (tune.ctas_per_sm > 0) occ = std::min(occ, tune.ctas_per_sm);
   occ = std::max(occ, 1);
   int64_t g = (int64_t)ctx->sm_count * occ;
   items = std::max(items, ceil_div(fitems * (1 + foot_stat), (int64_t)foot_chunk * (kRowsThreads / 32)));
   g = std::min<int64_t>(g, std::max<int64_t>(items, 1));
   return (int)g;
+}
+
+// The pass's row-walk and closed-form items: one launch, or one for each kind (`apart`).
+int ws_plan::enqueue_rows(const EnumArgs &args, bool apart, cudaStream_t st, int *launches) {
+  EnumArgs ea = args;
+  int64_t items = ea.ritem_hi - ea.ritem_lo;
+  const int64_t fitems = ea.fitem_hi - ea.fitem_lo;
+  if (apart) {
+    ea.fitem_hi = ea.fitem_lo;
+    CU(launch_rows(ea, grid_rows(items, 0), st));
+    ++*launches;
+    ea.fitem_hi = args.fitem_hi;
+    ea.ritem_lo = ea.ritem_hi;
+    items = 0;
+  }
+  if (items > 0 || fitems > 0) {
+    CU(launch_rows(ea, grid_rows(items, fitems), st));
+    ++*launches;
+  }
+  return WS_OK;
 }
 
 int ws_plan::grid_for(int threads, int64_t items, bool counting) const {
@@ -1844,10 +1876,7 @@ int ws_plan::enqueue(cudaStream_t st, std::vector<cudaEvent_t> *ev, ws_profile *
       ++launches;
     }
     if ((rc = mark(1 + 3 * (int)p)) != WS_OK) return rc;
-    if (P.ritem_hi > P.ritem_lo || P.fitem_hi > P.fitem_lo) {
-      CU(launch_rows(ea, grid_rows(P.ritem_hi - P.ritem_lo, P.fitem_hi - P.fitem_lo), st));
-      ++launches;
-    }
+    if ((rc = enqueue_rows(ea, P.apart, st, &launches)) != WS_OK) return rc;
     if ((rc = mark(2 + 3 * (int)p)) != WS_OK) return rc;
     CountArgs ca;
     ca.fld = ea.fld;
@@ -1963,7 +1992,9 @@ int ws_plan::run_plain_launches(cudaStream_t st) {
       ea.bank_shift = bank_shift();
       ea.block_pairs = block_pairs;
       if (it_hi > it_lo) CU(launch_enum(ea, grid_for(tune.enum_threads, it_hi - it_lo, false), tune.enum_threads, st));
-      if (rt_hi > rt_lo || ft_hi > ft_lo) CU(launch_rows(ea, grid_rows(rt_hi - rt_lo, ft_hi - ft_lo), st));
+      int n = 0;
+      const int rc = enqueue_rows(ea, false, st, &n);
+      if (rc != WS_OK) return rc;
       CountArgs ca;
       ca.fld = ea.fld;
       ca.item_unit = ea.own_foot + fitem_begin_end;
