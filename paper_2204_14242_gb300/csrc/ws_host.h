@@ -145,6 +145,7 @@ struct ws_plan {
   std::vector<int64_t> grp_foot_cost;    // closed form: estimated warp instructions per field
   std::vector<int64_t> grp_slots;        // row slots of the group's candidate
   std::vector<int64_t> grp_blk_slots;    //   those of its representative block
+  std::vector<int64_t> grp_wave_slots;   //   those of its wave
   std::vector<ws::WarpClasses> grp_classes;  // block warp classes per group (used with the row walk)
   std::vector<int64_t> grp_winstr_rows;  // modelled (warp, instruction) pairs of levels 1-3
   // work-item sizes set by layout(): row slots per row-walk item (256, 512 or 1024),
@@ -162,12 +163,12 @@ struct ws_plan {
   std::vector<ws::DPass> passes;
   int64_t scratch_words = 0;
   size_t scratch_bytes = 0;
-  int64_t item_begin_end = 0, ritem_begin_end = 0, citem_begin_end = 0, fitem_begin_end = 0;
+  int64_t item_begin_end = 0, ritem_begin_end = 0, citem_begin_end = 0, fitem_begin_end = 0, sitem_begin_end = 0;
   // counting items of every bitmap the plan accounts scratch for; citem_begin_end are those of
   // the bitmaps it fills (levels counted in closed form fill none)
   int64_t citems_accounted = 0;
   int32_t foot_chunk = 1;        // closed-form items a warp takes at once
-  int32_t foot_stat = 1;         // items per group for what the closed-form walk does not count
+  int32_t foot_stat = 1;         // least items per group for what the closed-form walk does not count
   int64_t own_budget = 0;        // owner-table entries the descriptor estimate allows for
   size_t grab_bytes = 0, counters_bytes = 0;
   // uploaded arrays that the plan owns until it is destroyed (their copies are asynchronous)
@@ -195,7 +196,7 @@ struct ws_plan {
   void layout();
   int upload_fields(cudaStream_t st);
   int grid_for(int threads, int64_t items, bool counting) const;
-  int grid_rows(int64_t items, int64_t fitems) const;
+  int grid_rows(int64_t items, int64_t fitems, int64_t sitems) const;
   int enqueue_rows(const ws::EnumArgs &args, bool apart, cudaStream_t st, int *launches);
   int bank_shift() const;
   int enqueue(cudaStream_t st, std::vector<cudaEvent_t> *ev, ws_profile *prof);

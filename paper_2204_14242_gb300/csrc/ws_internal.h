@@ -189,8 +189,8 @@ struct DGroup {
   uint8_t levels;         // level mask of its fields (1 block, 2 wave + y / z, 3 both)
   uint8_t first_wave;     // the candidate's first group with wave work counts the wave LUPs
   uint8_t foot;           // closed-form footprints taken: 1 wave + y / z sets, 2 the representative block
-  uint8_t pad8;
-  int32_t f_parts;        // closed-form items per counted field (parts of its target rows)
+  uint8_t f_parts;        // closed-form items per counted field (parts of its target rows)
+  int32_t s_parts;        // items for what the closed-form walk does not count (foot & 1)
   uint32_t foot_fields;   // the fields counted (bit k: the group's k-th), the others being moved copies of them
   int32_t n_loads;        // folded loads of all its fields
   int32_t n_stores;       // folded stores of all its fields
@@ -203,6 +203,7 @@ struct DGroup {
   int32_t n_rep;
   uint8_t rep_warp[32];
   uint8_t rep_mult[32];
+  int32_t sitem_begin;    // the first of those s_parts items
   int64_t fitem_begin;    // first closed-form item (field-major, f_parts per counted field)
 };
 
@@ -218,6 +219,7 @@ struct DPass {
   int64_t item_lo, item_hi;    // enumeration items of the pass
   int64_t ritem_lo, ritem_hi;  // row-walk items of the pass
   int64_t fitem_lo, fitem_hi;  // closed-form items of the pass
+  int64_t sitem_lo, sitem_hi;  // items for what the closed-form walk does not count
   int64_t citem_lo, citem_hi;  // counting items of the pass
   int32_t cf_lo, cf_hi;        // (candidate, field) index range
   int32_t grp_lo, grp_hi;      // field-group index range

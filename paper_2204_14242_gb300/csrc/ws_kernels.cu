@@ -2003,7 +2003,7 @@ __device__ __noinline__ void foot_field(const EnumArgs &a, FootSmem &m, const DF
 }
 
 // The closed-form items of a pass: warps take fchunk consecutive ones at a time and keep the
-// geometry of a field group while they stay in it; before them fstat items per group for
+// geometry of a field group while they stay in it; before them each group's s_parts items for
 // what the walk does not count.
 __device__ __forceinline__ void foot_items(const EnumArgs &a, FootSmem &m) {
   const uint32_t lane = threadIdx.x & 31u;
@@ -2013,16 +2013,16 @@ __device__ __forceinline__ void foot_items(const EnumArgs &a, FootSmem &m) {
     unsigned long long i0 = 0;
     if (lane == 0) i0 = atomicAdd(a.fgrab, (unsigned long long)a.fchunk);
     const int64_t it0 = a.fitem_lo + (int64_t)__shfl_sync(FULL, i0, 0);
-    const int64_t ns = (int64_t)(a.grp_hi - a.grp_lo) * a.fstat;
+    const int64_t ns = a.sitem_hi - a.sitem_lo;
     const int64_t it_end = a.fitem_hi + ns;
-    if (it0 >= it_end || a.fitem_hi == a.fitem_lo) break;
+    if (it0 >= it_end) break;
     const int64_t it1 = min(it0 + a.fchunk, it_end);
 #pragma unroll 1
     for (int64_t it = it0; it < it1; ++it) {
       if (it < a.fitem_lo + ns) {
-        const int i = (int)(it - a.fitem_lo), gi = i / a.fstat;
-        const DGroup &G = a.grp[a.grp_lo + gi];
-        if (G.foot & 1) foot_stats(a, G, m.sreq, i - gi * a.fstat, a.fstat);
+        const int64_t s = a.sitem_lo + (it - a.fitem_lo);
+        const DGroup &G = a.grp[a.own_stat[s]];
+        foot_stats(a, G, m.sreq, (int)(s - G.sitem_begin), G.s_parts);
         continue;
       }
       const int64_t itf = it - ns;

@@ -24,9 +24,9 @@ struct EnumArgs {
   int64_t ritem_lo, ritem_hi;      // row-walk items of the pass
   const int32_t *own_foot;         // field group of every closed-form item
   int64_t fitem_lo, fitem_hi;      // closed-form items of the pass
+  const int32_t *own_stat;         // field group of every item for what the closed-form walk does not count
+  int64_t sitem_lo, sitem_hi;      // those of the pass
   int32_t fchunk;                  // closed-form items a warp takes at once
-  int32_t fstat;                   // items per group for what the closed-form walk does not count
-  int32_t grp_lo, grp_hi;          // field groups of the pass
   int32_t chunk;                   // modelled warps per item
   int32_t chunk_rows;              // row slots per item (row walk)
   int32_t banks, bank_bytes, pair_dist;

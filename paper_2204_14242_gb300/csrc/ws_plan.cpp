@@ -1444,6 +1444,13 @@ static constexpr double kApartRatio = 0.35;
 static constexpr int64_t kFootUnitMin = 1000, kFootUnitSmall = 10000, kFootUnitMax = 32000, kFootParts = 64,
                          kFootPerWarp = 3;
 
+// What the closed-form walk does not count of a group (foot_stats) goes over the row slots of its wave, some
+// 0.5 us for 32 of them in one warp.  Up to eight items a group where there are few groups, and as many as
+// share the plan's slots out four to a resident warp, of at least kStatSlotsMin (the plain form: just that)
+// and at most kStatSlotsMax slots: with eight items whatever the wave, one 7-point candidate with a wave of 400,000
+// blocks of 4 x 8 x 4 took 228 us a step, now 93; 4,000 mixed candidates 2.27 and 2.23 ms (GB300).
+static constexpr int64_t kStatSlotsMin = 256, kStatSlotsMax = 8192;
+
 // Numbers work items and cuts passes for the current tuning.
 // Runs fn(lo, hi) over [0, n) in chunks on the host pool (defined with the pool below).
 static void parallel_chunks(int64_t n, int64_t chunk, const std::function<void(int64_t, int64_t)> &fn);
@@ -1523,7 +1530,7 @@ void ws_plan::layout() {
   // closed-form items: a field's units are shared out among parts of foot_unit estimated warp
   // instructions (kFootPerWarp and its neighbours; two CTAs of eight warps are resident per SM),
   // without exceeding the owner-table entries the descriptor estimate allowed for
-  int64_t foot_unit = kFootUnitMin;
+  int64_t foot_unit = kFootUnitMin, stat_slots = kStatSlotsMax;
   {
     const int64_t warps = 16 * (int64_t)(ctx ? ctx->sm_count : 152);
     int64_t cost = 0, fields = 0;
@@ -1541,7 +1548,12 @@ void ws_plan::layout() {
     foot_chunk = (int32_t)std::max<int64_t>(1, std::min<int64_t>(8, fields / (64 * warps)));
     if (plain_layout) foot_chunk = 1;
     int foot_groups = 0;
-    for (int g = 0; g < ng; ++g) foot_groups += hgrp[(size_t)g].foot != 0;
+    int64_t wave_slots = 0;
+    for (int g = 0; g < ng; ++g) {
+      foot_groups += hgrp[(size_t)g].foot != 0;
+      if (hgrp[(size_t)g].foot & 1) wave_slots += grp_wave_slots[(size_t)g];
+    }
+    stat_slots = plain_layout ? kStatSlotsMin : std::max(kStatSlotsMin, std::min(kStatSlotsMax, wave_slots / (4 * warps)));
     const int64_t share = 4 * warps / std::max<int64_t>(1, plain_layout ? 1 : foot_groups);
     foot_stat = (int32_t)std::max<int64_t>(1, std::min<int64_t>(8, share));
   }
@@ -1551,7 +1563,7 @@ void ws_plan::layout() {
   // chunks of the remaining modelled warps, or, for the row walk, chunks of row slots
   std::vector<int64_t> gbase((size_t)ng, 0);
   std::vector<int32_t> gpass((size_t)ng, 0);
-  int64_t items = 0, ritems = 0, fitems = 0;
+  int64_t items = 0, ritems = 0, fitems = 0, sitems = 0;
   {
     DPass cur;
     memset(&cur, 0, sizeof(cur));
@@ -1563,6 +1575,7 @@ void ws_plan::layout() {
       cur.item_hi = items;
       cur.ritem_hi = ritems;
       cur.fitem_hi = fitems;
+      cur.sitem_hi = sitems;
       cur.words = used;
       cur.apart = foot_work > 0 && walk_work >= kApartWork && (double)walk_work >= kApartRatio * (double)foot_work;
       walk_work = foot_work = 0;
@@ -1576,6 +1589,7 @@ void ws_plan::layout() {
         cur.item_lo = items;
         cur.ritem_lo = ritems;
         cur.fitem_lo = fitems;
+        cur.sitem_lo = sitems;
         cur.cf_lo = G.f_begin;
         cur.grp_lo = g;
         used = 0;
@@ -1589,8 +1603,11 @@ void ws_plan::layout() {
                                   : 0;
       items += G.n0_items;
       G.fitem_begin = fitems;
-      G.f_parts = G.foot ? (int32_t)std::max<int64_t>(1, std::min<int64_t>(kFootParts, grp_foot_cost[(size_t)g] / foot_unit)) : 0;
+      G.f_parts = G.foot ? (uint8_t)std::max<int64_t>(1, std::min<int64_t>(kFootParts, grp_foot_cost[(size_t)g] / foot_unit)) : 0;
       fitems += (int64_t)__builtin_popcount(G.foot_fields) * G.f_parts;
+      G.sitem_begin = (int32_t)sitems;
+      G.s_parts = G.foot & 1 ? (int32_t)std::max<int64_t>(foot_stat, ceil_div(grp_wave_slots[(size_t)g], stat_slots)) : 0;
+      sitems += G.s_parts;
       walk_work += row_slots(g) * (G.n_iv + G.n_stores);
       if (G.foot) foot_work += grp_foot_cost[(size_t)g] * __builtin_popcount(G.foot_fields);
       if (G.rows) ritems += ceil_div(row_slots(g), chunk_rows());
@@ -1602,7 +1619,7 @@ void ws_plan::layout() {
   // two), so that none of them is left for the end
   if (!plain_layout) {
     auto bucket = [&](int g) {
-      const int64_t c = grp_foot_cost[(size_t)g] / std::max(1, hgrp[(size_t)g].f_parts);
+      const int64_t c = grp_foot_cost[(size_t)g] / std::max<int64_t>(1, hgrp[(size_t)g].f_parts);
       return c > 0 ? __builtin_clzll((unsigned long long)c) : 64;
     };
     for (const DPass &P : passes) {
@@ -1723,9 +1740,10 @@ void ws_plan::layout() {
   ritem_begin_end = ritems;
   citem_begin_end = citems;
   fitem_begin_end = fitems;
-  // owners of the items: [enumeration | row walk | closed form], then the counting items' first
-  // units (with an end), then the counting units as (field, chunk) pairs
-  own.resize((size_t)(items + ritems + fitems + citems + 1) + cunits_.size());
+  sitem_begin_end = sitems;
+  // owners of the items: [enumeration | row walk | closed form | what that does not count], then the
+  // counting items' first units (with an end), then the counting units as (field, chunk) pairs
+  own.resize((size_t)(items + ritems + fitems + sitems + citems + 1) + cunits_.size());
   parallel_chunks(ng, 1024, [&](int64_t lo, int64_t hi) {
     for (int64_t g = lo; g < hi; ++g) {
       const DGroup &G = hgrp[(size_t)g];
@@ -1735,9 +1753,10 @@ void ws_plan::layout() {
       std::fill(own.begin() + items + G.ritem_begin, own.begin() + items + r1, (int32_t)g);
       std::fill_n(own.begin() + items + ritems + G.fitem_begin, (int64_t)__builtin_popcount(G.foot_fields) * G.f_parts,
                   (int32_t)g);
+      std::fill_n(own.begin() + items + ritems + fitems + G.sitem_begin, G.s_parts, (int32_t)g);
     }
   });
-  const int64_t at = items + ritems + fitems;
+  const int64_t at = items + ritems + fitems + sitems;
   std::copy(citem_unit_.begin(), citem_unit_.end(), own.begin() + at);
   own[(size_t)(at + citems)] = (int32_t)units;
   std::copy(cunits_.begin(), cunits_.end(), own.begin() + at + citems + 1);
@@ -1783,13 +1802,14 @@ int ws_plan::bank_shift() const {
 
 // CTAs of rows_kernel (of its instance without closed-form items where there are none): one per
 // row-walk item, one per eight warps' closed-form items.
-int ws_plan::grid_rows(int64_t items, int64_t fitems) const {
+int ws_plan::grid_rows(int64_t items, int64_t fitems, int64_t sitems) const {
   int occ = 1;
   rows_occupancy(iv_cap, fitems > 0, &occ);
   if (tune.ctas_per_sm > 0) occ = std::min(occ, tune.ctas_per_sm);
   occ = std::max(occ, 1);
   int64_t g = (int64_t)ctx->sm_count * occ;
-  items = std::max(items, ceil_div(fitems * (1 + foot_stat), (int64_t)foot_chunk * (kRowsThreads / 32)));
+  const int64_t witems = std::max(fitems * (1 + foot_stat), fitems + sitems);
+  items = std::max(items, ceil_div(witems, (int64_t)foot_chunk * (kRowsThreads / 32)));
   g = std::min<int64_t>(g, std::max<int64_t>(items, 1));
   return (int)g;
 }
@@ -1801,14 +1821,14 @@ int ws_plan::enqueue_rows(const EnumArgs &args, bool apart, cudaStream_t st, int
   const int64_t fitems = ea.fitem_hi - ea.fitem_lo;
   if (apart) {
     ea.fitem_hi = ea.fitem_lo;
-    CU(launch_rows(ea, grid_rows(items, 0), st));
+    CU(launch_rows(ea, grid_rows(items, 0, 0), st));
     ++*launches;
     ea.fitem_hi = args.fitem_hi;
     ea.ritem_lo = ea.ritem_hi;
     items = 0;
   }
   if (items > 0 || fitems > 0) {
-    CU(launch_rows(ea, grid_rows(items, fitems), st));
+    CU(launch_rows(ea, grid_rows(items, fitems, ea.sitem_hi - ea.sitem_lo), st));
     ++*launches;
   }
   return WS_OK;
@@ -1855,13 +1875,13 @@ int ws_plan::enqueue(cudaStream_t st, std::vector<cudaEvent_t> *ev, ws_profile *
     ea.own_rows = ea.own_enum + item_begin_end;
     ea.own_foot = ea.own_rows + ritem_begin_end;
     ea.fchunk = foot_chunk;
-    ea.fstat = foot_stat;
+    ea.own_stat = ea.own_foot + fitem_begin_end;
+    ea.sitem_lo = P.sitem_lo;
+    ea.sitem_hi = P.sitem_hi;
     ea.ritem_lo = P.ritem_lo;
     ea.ritem_hi = P.ritem_hi;
     ea.fitem_lo = P.fitem_lo;
     ea.fitem_hi = P.fitem_hi;
-    ea.grp_lo = P.grp_lo;
-    ea.grp_hi = P.grp_hi;
     ea.item_lo = P.item_lo;
     ea.item_hi = P.item_hi;
     ea.chunk = tune.chunk_warps;
@@ -1880,7 +1900,7 @@ int ws_plan::enqueue(cudaStream_t st, std::vector<cudaEvent_t> *ev, ws_profile *
     if ((rc = mark(2 + 3 * (int)p)) != WS_OK) return rc;
     CountArgs ca;
     ca.fld = ea.fld;
-    ca.item_unit = ea.own_foot + fitem_begin_end;
+    ca.item_unit = ea.own_stat + sitem_begin_end;
     ca.units = ca.item_unit + citem_begin_end + 1;
     ca.scratch = ea.scratch;
     ca.counters = ea.counters;
@@ -1975,15 +1995,15 @@ int ws_plan::run_plain_launches(cudaStream_t st) {
       ea.own_rows = ea.own_enum + item_begin_end;
       ea.own_foot = ea.own_rows + ritem_begin_end;
       ea.fchunk = foot_chunk;
-      ea.fstat = foot_stat;
+      ea.own_stat = ea.own_foot + fitem_begin_end;
+      ea.sitem_lo = hgrp[glo].sitem_begin;
+      ea.sitem_hi = ghi < ng ? hgrp[ghi].sitem_begin : sitem_begin_end;
       ea.item_lo = it_lo;
       ea.item_hi = it_hi;
       ea.ritem_lo = rt_lo;
       ea.ritem_hi = rt_hi;
       ea.fitem_lo = ft_lo;
       ea.fitem_hi = ft_hi;
-      ea.grp_lo = glo;
-      ea.grp_hi = ghi;
       ea.chunk = tune.chunk_warps;
       ea.chunk_rows = chunk_rows();
       ea.banks = hw.banks;
@@ -1997,7 +2017,7 @@ int ws_plan::run_plain_launches(cudaStream_t st) {
       if (rc != WS_OK) return rc;
       CountArgs ca;
       ca.fld = ea.fld;
-      ca.item_unit = ea.own_foot + fitem_begin_end;
+      ca.item_unit = ea.own_stat + sitem_begin_end;
       ca.units = ca.item_unit + citem_begin_end + 1;
       ca.scratch = ea.scratch;
       ca.counters = counters;
@@ -2414,7 +2434,7 @@ struct ClosedFormCost {
 struct GroupOut {
   std::vector<DGroup> g;
   std::vector<char> iv_ok, rows_ok, foot_ok;
-  std::vector<int64_t> slots, blk_slots, winstr, foot_cost;
+  std::vector<int64_t> slots, blk_slots, wave_slots, winstr, foot_cost;
   std::vector<WarpClasses> cls;
   int32_t iv_cap = 0;
 };
@@ -2541,6 +2561,7 @@ static void build_groups(Plan *p, int i, const Compiled &cc, const ws_hw &hw, Gr
     go.foot_cost.push_back(foot ? (int64_t)cost_of.of(G.levels, stores, nd, reach, z_moved) : 0);
     // with the block level when the group also serves the representative block
     go.slots.push_back(dc.rows_slot_end[(G.levels & 1) ? 3 : 2]);
+    go.wave_slots.push_back(dc.rows_slot_end[0]);
     go.blk_slots.push_back((G.levels & 1) ? dc.rows_slot_end[3] - dc.rows_slot_end[2] : 0);
     {
       const DField &f0 = p->hfld[G.f_begin], &c0 = p->hfld[a];
@@ -2745,6 +2766,7 @@ static void build_host(Plan *p, const ws_config *cfgs, int n_cfg, const ws_field
   p->grp_foot_cost.reserve(ng);
   p->grp_slots.reserve(ng);
   p->grp_blk_slots.reserve(ng);
+  p->grp_wave_slots.reserve(ng);
   p->grp_classes.reserve(ng);
   p->grp_winstr_rows.reserve(ng);
   for (GroupOut &go : gout) {
@@ -2755,6 +2777,7 @@ static void build_host(Plan *p, const ws_config *cfgs, int n_cfg, const ws_field
     p->grp_foot_cost.insert(p->grp_foot_cost.end(), go.foot_cost.begin(), go.foot_cost.end());
     p->grp_slots.insert(p->grp_slots.end(), go.slots.begin(), go.slots.end());
     p->grp_blk_slots.insert(p->grp_blk_slots.end(), go.blk_slots.begin(), go.blk_slots.end());
+    p->grp_wave_slots.insert(p->grp_wave_slots.end(), go.wave_slots.begin(), go.wave_slots.end());
     p->grp_classes.insert(p->grp_classes.end(), go.cls.begin(), go.cls.end());
     p->grp_winstr_rows.insert(p->grp_winstr_rows.end(), go.winstr.begin(), go.winstr.end());
     p->iv_cap = std::max(p->iv_cap, go.iv_cap);
@@ -2984,7 +3007,7 @@ extern "C" int ws_plan_profile(ws_plan *p, void *stream, ws_profile *out) {
     out->ms_rank = ms;
     cudaEventElapsedTime(&ms, ev[0], ev[2 + 3 * np]);
     out->ms_total = ms;
-    out->enum_items = p->item_begin_end + p->ritem_begin_end + p->fitem_begin_end;
+    out->enum_items = p->item_begin_end + p->ritem_begin_end + p->fitem_begin_end + p->sitem_begin_end;
     out->count_items = p->citem_begin_end;
     out->passes = (int64_t)p->passes.size();
     out->upload_bytes = p->upload_bytes;
@@ -3374,7 +3397,7 @@ extern "C" int ws_plan_dry_run(const ws_config *cfgs, int n_cfg, const ws_field 
   out->groups = (int64_t)p.hgrp.size();
   out->passes = (int64_t)p.passes.size();
   out->enum_items = p.item_begin_end;
-  out->row_items = p.ritem_begin_end + p.fitem_begin_end;
+  out->row_items = p.ritem_begin_end + p.fitem_begin_end + p.sitem_begin_end;
   out->count_items = p.citems_accounted;
   out->access_entries = (int64_t)h.hacc.size();
   out->interval_entries = (int64_t)h.hiv.size();
