@@ -667,6 +667,8 @@ struct RowsPerPlane {
 //    to spare in two pitches, so that they reach no further than the next row's cell;
 //  * within a level's class of runs the ranges overlap or touch: the offsets' rests are spread by
 //    at most the shortest run and one sector;
+//  * row numbers stay in 32 bits: a task's target rows, R of the level and `reach` of the
+//    displacements, and two planes behind them (where the kernel's planes end), are below 2^31;
 //  * the wave holds fewer than 2^32 sectors: the counts of an item are 32-bit sums.  At most that
 //    many are the sectors of the address range, and the accesses its threads issue (touched: one
 //    sector each; the y and z sets are parts of the wave moved).  64-bit sums need no such limit,
@@ -687,21 +689,26 @@ static void closed_form_ok(const ws_field &F, const FieldFold &ff, int mask, con
     rows = {F.stride[1], F.stride[2], F.stride[2] / F.stride[1], {}};
     if (rows.q * F.stride[1] != F.stride[2]) rows.q = 0;
   }
+  // rows from the lowest displacement (or none) to the highest (each list is sorted)
+  int64_t dmin = 0, dmax = 0;
+  for (int ls = 0, e = ff.n_iv; ls < 2; e += ff.n_dsp[ls++]) {
+    if (ff.n_dsp[ls] == 0) continue;
+    DDsp a, b;
+    memcpy(&a, &ff.iv[(size_t)e], sizeof(a));
+    memcpy(&b, &ff.iv[(size_t)(e + ff.n_dsp[ls] - 1)], sizeof(b));
+    dmin = std::min<int64_t>(dmin, a.d);
+    dmax = std::max<int64_t>(dmax, b.d);
+  }
+  const int64_t reach = dmax - dmin;
   int64_t q = rows.q;
   const bool planes = q >= ny && q < ((int64_t)1 << 30);   // the displacements' rows within a plane are known
   if (!planes) {
     // the level lies in one plane: all its target rows as those of one plane
     if (nz > 1) return;
-    int64_t dmin = 0, dmax = 0;
-    for (size_t e = (size_t)ff.n_iv; e < ff.iv.size(); ++e) {
-      DDsp d;
-      memcpy(&d, &ff.iv[e], sizeof(d));
-      dmin = std::min<int64_t>(dmin, d.d);
-      dmax = std::max<int64_t>(dmax, d.d);
-    }
-    q = ny + dmax - dmin + 2;
+    q = ny + reach + 2;
   }
-  if ((nz - 1) * q + ny >= ((int64_t)1 << 30) || q >= ((int64_t)1 << 30)) return;
+  const int64_t R = (nz - 1) * q + ny;
+  if (R >= ((int64_t)1 << 30) || q >= ((int64_t)1 << 30) || R + reach + 2 * q >= ((int64_t)1 << 31)) return;
   df.q = (int32_t)q;
   if (rows.fq.d != (uint32_t)q) rows.fq = make_fastdiv((uint32_t)q);
   df.fq_m = rows.fq.m;

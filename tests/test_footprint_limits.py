@@ -1,11 +1,15 @@
-"""Where the closed form of the footprints ends: waves of 2^32 sectors and more.
+"""Where the closed form of the footprints ends: 2^32 sectors, and row numbers of 32 bits.
 
 A closed-form item sums its counts in 32 bits, so a field whose wave may hold 2^32 sectors or more
-takes the address walk.  The arrays here are dense and aligned, one element a sector, and their
-waves cover the whole domain: the counts follow from the number of points alone.
+takes the address walk.  The arrays of those tests are dense and aligned, one element a sector, and
+their waves cover the whole domain: the counts follow from the number of points alone.
+
+Target rows are numbered in 32 bits, too, up to two planes behind the last one: where planes lie
+so far apart that these numbers do not fit, the address walk is taken.
 """
 import pytest
 
+import oracle
 from paper_2204_14242_gb300 import binding as B
 from paper_2204_14242_gb300 import workloads as W
 
@@ -56,3 +60,42 @@ def test_counts_beyond_32_bits(cfg, behind):
     assert (got["wave_store_sectors"], got["wave_store_lines"], got["wave_store_req_sectors"]) == (n, n // 4, n)
     assert (got["wave_load_sectors"], got["wave_load_lines"]) == (loads, loads // 4)
     assert got["ov_y"] == got["ov_z"] == got["y_lines"] == got["z_lines"] == 0
+
+
+def far(N, row, q):
+    """Loads of 8-byte elements in rows of 256 bytes, q rows a plane, `row` rows from the point."""
+    return W.Config(N=N, B=(8, 2, 1), fields=[W.Field(8, [W.Access(0, 0, 0, 0, 32 * row)], strides=(1, 32, 32 * q))],
+                    flops_per_lup=1.0, wave_blocks_override=1 << 20)
+
+
+FAR_Q = (1 << 30) - (1 << 21)
+FAR = [
+    (far((32, 4, 2), 5, FAR_Q // 2), True),
+    (far((32, 4, 2), (1 << 28) - 2, 1 << 28), True),
+    (far((32, 4, 1), (1 << 28) - 2, FAR_Q), True),           # one plane: the rows to the next do not matter
+    (far((32, 4, 2), 5, FAR_Q), False),
+    (far((32, 4, 2), (1 << 28) - 2, FAR_Q), False),          # target rows 2^28 - 2 .. and two planes from there
+    (far((32, 4, 2), 2 - (1 << 28), FAR_Q), False),
+]
+
+
+@pytest.mark.parametrize("cfg,closed", FAR)
+def test_far_rows_leave_the_closed_form(cfg, closed):
+    plan = B.ws_plan_dry_run([cfg], W.a100())
+    assert plan["candidates_ok"] == 1
+    assert (plan["row_items"] > 0) == closed
+
+
+@pytest.mark.gpu
+def test_far_rows_match_oracle():
+    cfgs = [c for c, _ in FAR]
+    want = oracle.estimate(cfgs, W.a100())
+    ctx = B.Context(0, 12 << 30)
+    try:
+        res, _ = B.ws_estimate_batch(ctx, cfgs, W.a100())
+    finally:
+        ctx.close()
+    for i, (got, w) in enumerate(zip(B.results_to_dicts(res), want)):
+        assert got["status"] == w["status"] == B.WS_OK
+        for k in B.RESULT_INT:
+            assert got[k] == w[k], (i, k, got[k], w[k])
