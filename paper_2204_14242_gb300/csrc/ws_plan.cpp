@@ -286,6 +286,7 @@ struct Compiled {
   std::pmr::vector<uint64_t> fkey;  // (field index, folding): equal keys have equal access lists
   std::pmr::vector<int64_t> need_words;  // bitmap words per field
   size_t dsc_bytes = 0;             // descriptor bytes of its fields, lists and groups
+  size_t dsp_bytes = 0;             // bytes of their displacements
   size_t need_sum = 0, need_max = 0;  // bitmap bytes of all its fields / of its largest
   size_t items_est = 0;             // bound on its work items (owner table entries)
   int64_t n_acc_own = 0, n_iv_own = 0;  // list entries of its fields that no other candidate shares
@@ -2343,7 +2344,7 @@ static void compile_all(const ws_config *cfgs, int n_cfg, const ws_field *fld, i
         const size_t cr = 256;   // the smallest row-walk item
         for (size_t k = 0; k < cc.f.size(); ++k) {
           const int64_t nacc = cc.acc_off[k + 1] - cc.acc_off[k], niv = cc.iv_off[k + 1] - cc.iv_off[k];
-          // (the displacements of the closed form: see descriptor_extra)
+          cc.dsp_bytes += (size_t)(cc.f[k].n_dsp_l + cc.f[k].n_dsp_s) * sizeof(DDsp);   // (descriptor_extra)
           cc.dsc_bytes += sizeof(DField) + sizeof(DGroup) + (size_t)nacc * sizeof(DAcc) +
                           (size_t)cc.f[k].n_iv * sizeof(DIv);
           cc.need_sum += (size_t)cc.need_words[k] * 4;
@@ -2599,22 +2600,19 @@ constexpr size_t kDescHeadroom = (size_t)8 << 20;
 // given arena without them still does.
 static size_t descriptor_extra(const CompileArena &ca, const std::vector<int> &status) {
   const size_t room = kDescHeadroom - ((size_t)256 << 10);   // (the rest: granularity of the buffers)
-  std::unordered_set<uint64_t> seen;
   size_t bytes = 0;
-  for (int once = 0; once < 2; ++once) {   // every field's list, then (seldom) shared ones once
-    bytes = 0;
-    for (size_t i = 0; i < status.size(); ++i) {
-      if (status[i] != WS_OK) continue;
-      const Compiled &cc = *ca.comp[i];
-      for (size_t k = 0; k < cc.f.size(); ++k) {
-        bytes += kGrabBytes;
-        if (!once || cc.fkey[k] == kNoShare || seen.insert(cc.fkey[k]).second)
-          bytes += (size_t)(cc.f[k].n_dsp_l + cc.f[k].n_dsp_s) * sizeof(DDsp);
-      }
-    }
-    if (bytes <= room) return 0;
+  for (size_t i = 0; i < status.size(); ++i)
+    if (status[i] == WS_OK) bytes += ca.comp[i]->dsp_bytes + kGrabBytes * ca.comp[i]->f.size();
+  if (bytes <= room) return 0;
+  std::unordered_set<uint64_t> seen;   // (seldom) the shared lists once
+  for (size_t i = 0; i < status.size(); ++i) {
+    if (status[i] != WS_OK || !ca.comp[i]->any_shared) continue;
+    const Compiled &cc = *ca.comp[i];
+    for (size_t k = 0; k < cc.f.size(); ++k)
+      if (cc.fkey[k] != kNoShare && !seen.insert(cc.fkey[k]).second)
+        bytes -= (size_t)(cc.f[k].n_dsp_l + cc.f[k].n_dsp_s) * sizeof(DDsp);
   }
-  return bytes - room;
+  return bytes > room ? bytes - room : 0;
 }
 
 static void build_host(Plan *p, const ws_config *cfgs, int n_cfg, const ws_field *fld, int n_fld,
