@@ -1661,9 +1661,12 @@ void ws_plan::layout() {
   auto pack = [&](int64_t sg, bool write, int64_t item0, int64_t unit0) {
     bool open = false;
     int64_t n_items = 0, n_units = 0, pages_in = 0, units_in = 0;
-    int64_t a_items = 0, a_pages = 0, a_units = 0;   // the same with the units the closed form makes needless
+    // the same with the units the closed form makes needless: only a dry run reports them
+    int64_t a_items = 0, a_pages = 0, a_units = 0;
+    const bool account = ctx == nullptr;
     for (int g = seg_start[(size_t)sg]; g < seg_start[(size_t)sg + 1]; ++g) {
       const DGroup &G = hgrp[(size_t)g];
+      const bool closed = G.foot && G.foot == ((G.levels & 1 ? 2 : 0) | (G.levels & 2 ? 1 : 0));   // no bitmaps filled
       int64_t o = gbase[(size_t)g];
       for (int k = 0; k < G.f_count; ++k) {
         const int32_t fi = G.f_begin + k;
@@ -1690,14 +1693,17 @@ void ws_plan::layout() {
           f.item_begin = G.item_begin;
           f.citem_begin = item0 + n_items - (open ? 1 : 0);
         }
+        if (closed && !account) continue;
         const int64_t kb = ceil_div(f.words[0], G.rows ? (int64_t)kPagedChunkWords : (int64_t)tune.count_words);
         for_count_units(f, G.rows != 0, tune.count_words, [&](int64_t u, int64_t pages) {
-          if (a_items == 0 || a_pages + pages > kCountMaxPages || a_units == count_pack) {
-            ++a_items;
-            a_pages = a_units = 0;
+          if (account && !write) {
+            if (a_items == 0 || a_pages + pages > kCountMaxPages || a_units == count_pack) {
+              ++a_items;
+              a_pages = a_units = 0;
+            }
+            a_pages += pages;
+            ++a_units;
           }
-          a_pages += pages;
-          ++a_units;
           if (G.foot & (u < kb ? 2 : 1)) return;
           if (!open || pages_in + pages > kCountMaxPages || units_in == count_pack) {
             if (write) citem_unit_[(size_t)(item0 + n_items)] = (int32_t)(unit0 + n_units);
