@@ -371,7 +371,8 @@ static void field_displacements(const ws_field &F, FieldFold &out) {
   const __int128 P = (__int128)F.elem_bytes * F.stride[1];
   out.n_dsp[0] = out.n_dsp[1] = 0;
   out.dsp_spread[0] = out.dsp_spread[1] = 0;
-  out.dsp_ok = P > 0 && P <= ((int64_t)1 << 28);
+  const __int128 esx = (__int128)F.elem_bytes * F.stride[0];   // (closed_form_ok refuses any other)
+  out.dsp_ok = P > 0 && P <= ((int64_t)1 << 28) && esx >= 0 && esx <= 32;
   if (!out.dsp_ok) return;
   const int64_t p = (int64_t)P;
   const double inv = 1.0 / (double)p;
@@ -569,7 +570,8 @@ static void cover_runs(int fold_axis, int fold, FieldFold &out) {
   if (out.covered) return;
   out.covered = true;
   const std::vector<RunRow> &rr = out.rr;
-  std::vector<DIv> iv(out.iv.begin(), out.iv.begin() + out.n_iv);
+  std::vector<DIv> &iv = out.iv_cov;   // (its room is kept from field to field)
+  iv.assign(out.iv.begin(), out.iv.begin() + out.n_iv);
   // covering runs: order runs by (|dy| + |dz|, dz, dy); a run may be covered by an earlier
   // one of the same dc whose x offsets contain its own, at a row displacement a thread row
   // can make (a multiple of the fold along the folding axis); the nearest one is taken
@@ -632,7 +634,7 @@ static void cover_runs(int fold_axis, int fold, FieldFold &out) {
     for (int kd = 0; kd < 3; ++kd)
       for (const DIv &v : iv)
         if (kind(v) == kd) tmp.push_back(v);
-    iv.swap(tmp);
+    std::copy(tmp.begin(), tmp.end(), iv.begin());
   }
   out.n_iv_unc = out.n_iv_zc = 0;
   out.cov_dy = out.cov_dz = out.cov_dy_y = 0;
@@ -648,7 +650,6 @@ static void cover_runs(int fold_axis, int fold, FieldFold &out) {
     out.cov_dz = std::max<int16_t>(out.cov_dz, (int16_t)std::abs(v.ddz));
   }
   iv.insert(iv.end(), out.iv.begin() + out.n_iv, out.iv.end());
-  out.iv_cov.swap(iv);
 }
 
 // Rows from plane to plane of the field before (a candidate's fields mostly share them); no field
@@ -1230,10 +1231,13 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     if (has_l) need += df.words[0] + 3 * df.words[1];
     if (has_s) need += df.words[0] + df.words[1];
     need += page_flag_words(df.words[0], df.words[1]);   // used when the field takes the row walk
-    out.f.push_back(df);
     out.acc.insert(out.acc.end(), ff->da.begin(), ff->da.end());
     const std::vector<DIv> &iv = cover ? ff->iv_cov : ff->iv;
-    out.iv.insert(out.iv.end(), iv.begin(), iv.end());
+    // a refused field's displacements are not read (a shared list keeps them for its other fields)
+    const bool dsp = df.closed != 0 || key != kNoShare;
+    if (!dsp) df.n_dsp_l = df.n_dsp_s = 0;
+    out.f.push_back(df);
+    out.iv.insert(out.iv.end(), iv.begin(), dsp ? iv.end() : iv.begin() + ff->n_iv);
     out.acc_off.push_back((int32_t)out.acc.size());
     out.iv_off.push_back((int32_t)out.iv.size());
     out.fkey.push_back(key != kNoShare && cover ? key | kCoveredKey : key);

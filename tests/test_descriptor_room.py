@@ -47,6 +47,18 @@ def test_estimate_keeps_shared_lists_out():
     assert abs((d[2] - d[1]) - 18 * (d[1] - d[0])) <= 12 * (18 + 1)
 
 
+@pytest.mark.parametrize("z_extra,entries", [(0, 5 + 5 + 1), (1, 5)])
+def test_refused_fields_have_no_displacements(z_extra, entries):
+    """A 7-point field has five merged runs of loads, and in closed form displacements of five load
+    rows and one store row; planes that are no whole number of rows apart are refused."""
+    n, dims = 9, (64, 32, 32)
+    acc = [W.Access(*o) for o in W.star_offsets(1)] + [W.Access(0, 0, 0, 1)]
+    cfgs = [W.Config(N=dims, B=(32, 2, 1), fields=[W.Field(8, acc, strides=(1, 64, 64 * 32 + z_extra))],
+                     flops_per_lup=7.0, wave_blocks_override=200) for _ in range(n)]
+    plan = B.ws_plan_dry_run(cfgs, W.a100())
+    assert plan["candidates_ok"] == n and plan["interval_entries"] == n * entries
+
+
 @pytest.mark.gpu
 def test_small_arena_runs_in_passes():
     """The arena holds descriptors and some of the bitmaps: results as in one with room for all."""
