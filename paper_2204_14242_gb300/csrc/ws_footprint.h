@@ -26,27 +26,15 @@
 
 #include "ws_internal.h"
 
-#ifdef __CUDACC__
-#define WS_HD __host__ __device__ __forceinline__
-#define WS_HD_CALL static __host__ __device__ __noinline__
-#else
-#define WS_HD inline
-#define WS_HD_CALL inline
-#endif
+#define WS_FOOT __device__ __forceinline__
 
 namespace ws {
 
-WS_HD uint32_t foot_div(uint32_t n, uint32_t m, uint32_t s) {
-#ifdef __CUDA_ARCH__
-  return (__umulhi(n, m) + n) >> s;
-#else
-  return (uint32_t)((((uint64_t)n * m) >> 32) + n) >> s;
-#endif
-}
-WS_HD uint32_t foot_div(uint32_t n, const FastDiv &f) { return foot_div(n, f.m, f.s); }
-WS_HD int32_t foot_min(int32_t a, int32_t b) { return a < b ? a : b; }
-WS_HD int32_t foot_max(int32_t a, int32_t b) { return a > b ? a : b; }
-WS_HD uint32_t foot_umin(uint32_t a, uint32_t b) { return a < b ? a : b; }
+WS_FOOT uint32_t foot_div(uint32_t n, uint32_t m, uint32_t s) { return (__umulhi(n, m) + n) >> s; }
+WS_FOOT uint32_t foot_div(uint32_t n, const FastDiv &f) { return foot_div(n, f.m, f.s); }
+WS_FOOT int32_t foot_min(int32_t a, int32_t b) { return a < b ? a : b; }
+WS_FOOT int32_t foot_max(int32_t a, int32_t b) { return a > b ? a : b; }
+WS_FOOT uint32_t foot_umin(uint32_t a, uint32_t b) { return a < b ? a : b; }
 
 constexpr int32_t kRowInf = 0x7fffffff;   // no further state change
 constexpr int32_t kHullLo = 0x3fffffff, kHullHi = -0x3fffffff;   // an empty byte range
@@ -86,7 +74,7 @@ struct alignas(16) FootGeo {
 // Fills level l of g, in two steps so that lanes can share them: foot_level for each of the
 // three levels, then foot_finish.  Candidate c, rows q from plane to plane, esx >= 0 bytes from
 // point to point; the wave and its y and z sets, or the representative block alone.
-WS_HD void foot_level(FootGeo &g, const DCfg &c, int32_t q, int32_t esx, bool block, int l) {
+WS_FOOT void foot_level(FootGeo &g, const DCfg &c, int32_t q, int32_t esx, bool block, int l) {
   const int32_t gx = c.g[0], B0 = c.B[0], N0 = c.N[0];
   const int32_t lo = block ? (l == 0 ? (int32_t)c.rep : 0) : (int32_t)(l == 0 ? c.s : l == 1 ? c.y_lo : c.z_lo);
   const int32_t hi = block ? (l == 0 ? lo + 1 : 0) : (int32_t)(l == 0 ? c.s + c.weff : l == 1 ? c.y_hi : c.z_hi);
@@ -119,7 +107,7 @@ WS_HD void foot_level(FootGeo &g, const DCfg &c, int32_t q, int32_t esx, bool bl
   g.lev[l] = L;
 }
 
-WS_HD void foot_finish(FootGeo &g, const DCfg &c, int32_t q, int32_t esx) {
+WS_FOOT void foot_finish(FootGeo &g, const DCfg &c, int32_t q, int32_t esx) {
   const int32_t fy = c.fold_axis == 1 ? c.fold : 1, fz = c.fold_axis == 2 ? c.fold : 1;
   const int32_t gy = c.g[1], n2 = c.N[2], b1f = c.B[1] * fy, b2f = c.B[2] * fz;
   g.gy = gy;
@@ -165,7 +153,7 @@ WS_HD void foot_finish(FootGeo &g, const DCfg &c, int32_t q, int32_t esx) {
 // Byte ranges of one row, per level: [0] class P, [1] class S (empty: lo > hi).
 struct FootHull {
   int32_t lo[3][2], hi[3][2];
-  WS_HD void clear() {
+  WS_FOOT void clear() {
 #pragma unroll
     for (int l = 0; l < 3; ++l)
 #pragma unroll
@@ -185,7 +173,7 @@ struct FootRow {
 
 // Looks up row r (without branches: the lanes' rows differ).  Returns the next row at which the
 // state of a level may change (want_next; else anything).
-WS_HD int32_t foot_row(const FootGeo &g, int nl, int32_t r, bool want_next, FootRow &o) {
+WS_FOOT int32_t foot_row(const FootGeo &g, int nl, int32_t r, bool want_next, FootRow &o) {
   const int32_t zr = (int32_t)foot_div((uint32_t)r, g.fq_m, g.fq_s), row0 = zr * g.q;   // row0: the plane's first row
   const int32_t y = g.y0 + (r - row0), z = g.z0 + zr;
   const bool in = r >= 0 && z < g.z_end && y < g.n1;
@@ -218,7 +206,7 @@ WS_HD int32_t foot_row(const FootGeo &g, int nl, int32_t r, bool want_next, Foot
 }
 
 // Adds a row's runs, moved by [clo, chi], to h.
-WS_HD void foot_add(const FootRow &o, int nl, int32_t clo, int32_t chi, FootHull &h) {
+WS_FOOT void foot_add(const FootRow &o, int nl, int32_t clo, int32_t chi, FootHull &h) {
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
     if (l > 0 && nl == 1) break;
@@ -239,7 +227,7 @@ WS_HD void foot_add(const FootRow &o, int nl, int32_t clo, int32_t chi, FootHull
 // The two ranges of every level as one, [lo, hi].  Returns the levels present (bit l), and bit 3
 // where two ranges leave a gap between them (a start at most one sector behind an end leaves no
 // sector out): then one range will not do.
-WS_HD uint32_t foot_join(const FootHull &h, int nl, int32_t lo[3], int32_t hi[3]) {
+WS_FOOT uint32_t foot_join(const FootHull &h, int nl, int32_t lo[3], int32_t hi[3]) {
   uint32_t r = 0;
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
@@ -258,7 +246,7 @@ WS_HD uint32_t foot_join(const FootHull &h, int nl, int32_t lo[3], int32_t hi[3]
 
 // Planes from row r's target plane on (rows [r, r + q) move together) over which the states
 // repeat from plane to plane: up to the end of the blocks' slab, or of the levels.
-WS_HD int32_t foot_repeat(const FootGeo &g, int32_t r) {
+WS_FOOT int32_t foot_repeat(const FootGeo &g, int32_t r) {
   int32_t z = r >= 0 ? (int32_t)foot_div((uint32_t)r, g.fq_m, g.fq_s)
                      : -(int32_t)foot_div((uint32_t)(g.q - 1 - r), g.fq_m, g.fq_s);
   const int32_t yr = r - z * g.q;
@@ -276,7 +264,7 @@ WS_HD int32_t foot_repeat(const FootGeo &g, int32_t r) {
 }
 
 // Slab of plane z (from row 0's), -1 where no level has rows.
-WS_HD int32_t foot_slab(const FootGeo &g, int32_t z) {
+WS_FOOT int32_t foot_slab(const FootGeo &g, int32_t z) {
   const int32_t zz = z + g.z0;
   return z < 0 || zz >= g.z_end ? -1 : (int32_t)foot_div((uint32_t)zz, g.fb2_m, g.fb2_s);
 }
@@ -284,7 +272,7 @@ WS_HD int32_t foot_slab(const FootGeo &g, int32_t z) {
 // What rows r .. r + n - 1 (n <= q + 2) depend on: the row's place in its plane and the slabs of
 // the planes they touch with rows that hold points (-2: none touched).  Two displacements that
 // agree on these look up the same states throughout.  Returns whether any state can be present.
-WS_HD bool foot_key(const FootGeo &g, int32_t r, int32_t n, int32_t key[4]) {
+WS_FOOT bool foot_key(const FootGeo &g, int32_t r, int32_t n, int32_t key[4]) {
   const int32_t z = r >= 0 ? (int32_t)foot_div((uint32_t)r, g.fq_m, g.fq_s)
                            : -(int32_t)foot_div((uint32_t)(g.q - 1 - r), g.fq_m, g.fq_s);
   const int32_t yr = r - z * g.q;
@@ -306,18 +294,18 @@ struct FootCounts {
 struct SecRange {
   int32_t a, b;
 };
-WS_HD int32_t foot_len(const SecRange &r) { return r.b - r.a + 1; }
-WS_HD int32_t foot_lines(const SecRange &r) { return (r.b >> 2) - (r.a >> 2) + 1; }
-WS_HD int32_t foot_ov(const SecRange &p, const SecRange &q) {
+WS_FOOT int32_t foot_len(const SecRange &r) { return r.b - r.a + 1; }
+WS_FOOT int32_t foot_lines(const SecRange &r) { return (r.b >> 2) - (r.a >> 2) + 1; }
+WS_FOOT int32_t foot_ov(const SecRange &p, const SecRange &q) {
   return foot_max(foot_min(p.b, q.b) - foot_max(p.a, q.a) + 1, 0);
 }
-WS_HD SecRange foot_cut(const SecRange &p, const SecRange &q) {
+WS_FOOT SecRange foot_cut(const SecRange &p, const SecRange &q) {
   SecRange r{foot_max(p.a, q.a), foot_min(p.b, q.b)};
   if (r.a > r.b) r = {kSecLo, kSecHi};
   return r;
 }
 // Sectors of the byte range [lo, hi] relative to address A, cut to [c0, c1).
-WS_HD SecRange foot_clip(int32_t A, int32_t lo, int32_t hi, int32_t c0, int32_t c1) {
+WS_FOOT SecRange foot_clip(int32_t A, int32_t lo, int32_t hi, int32_t c0, int32_t c1) {
   SecRange r{kSecLo, kSecHi};
   if (lo <= hi) {
     const int32_t a = foot_max((A + lo) >> 5, c0), b = foot_min((A + hi) >> 5, c1 - 1);
@@ -326,19 +314,19 @@ WS_HD SecRange foot_clip(int32_t A, int32_t lo, int32_t hi, int32_t c0, int32_t 
   return r;
 }
 // Two ranges as two disjoint ones that do not touch (the second empty when they did).
-WS_HD void foot_merge(SecRange &p, SecRange &q) {
+WS_FOOT void foot_merge(SecRange &p, SecRange &q) {
   if (foot_max(p.a, q.a) <= foot_min(p.b, q.b) + 1) {
     p = {foot_min(p.a, q.a), foot_max(p.b, q.b)};
     q = {kSecLo, kSecHi};
   }
 }
 // Lines of two disjoint ranges that do not touch (they can still meet in one line).
-WS_HD int32_t foot_lines2(const SecRange &p, const SecRange &q) {
+WS_FOOT int32_t foot_lines2(const SecRange &p, const SecRange &q) {
   return foot_lines(p) + foot_lines(q) - foot_max(foot_min(p.b >> 2, q.b >> 2) - foot_max(p.a >> 2, q.a >> 2) + 1, 0);
 }
 
 // Cell of the target row at address A (pitch P): sectors [c0, c1).
-WS_HD void foot_cell(int32_t A, int32_t P, int32_t hmin, int32_t &c0, int32_t &c1) {
+WS_FOOT void foot_cell(int32_t A, int32_t P, int32_t hmin, int32_t &c0, int32_t &c1) {
   c0 = ((A + hmin) >> 7) << 2;
   c1 = ((A + P + hmin) >> 7) << 2;
 }
@@ -346,7 +334,7 @@ WS_HD void foot_cell(int32_t A, int32_t P, int32_t hmin, int32_t &c0, int32_t &c
 // Counts one cell `mult` times when every level has at most one range per row: lo / hi are those
 // of the row (cur) and of the row before it (prv); bit l of `levels`: level l may be present, bit 4:
 // the z set's lines are wanted.
-WS_HD void foot_count(const int32_t clo[3], const int32_t chi[3], const int32_t plo[3], const int32_t phi[3],
+WS_FOOT void foot_count(const int32_t clo[3], const int32_t chi[3], const int32_t plo[3], const int32_t phi[3],
                       int32_t A, int32_t P, int32_t hmin, uint32_t mult, uint32_t levels, FootCounts &out) {
   int32_t c0, c1;
   foot_cell(A, P, hmin, c0, c1);
@@ -386,7 +374,7 @@ WS_HD void foot_count(const int32_t clo[3], const int32_t chi[3], const int32_t 
 }
 
 // Lines of the first level's cell alone.
-WS_HD uint32_t foot_count_lines(int32_t clo, int32_t chi, int32_t plo, int32_t phi, int32_t A, int32_t P, int32_t hmin) {
+WS_FOOT uint32_t foot_count_lines(int32_t clo, int32_t chi, int32_t plo, int32_t phi, int32_t A, int32_t P, int32_t hmin) {
   int32_t c0, c1;
   foot_cell(A, P, hmin, c0, c1);
   SecRange p = foot_clip(A - P, plo, phi, c0, c1), q = foot_clip(A, clo, chi, c0, c1);
@@ -396,7 +384,7 @@ WS_HD uint32_t foot_count_lines(int32_t clo, int32_t chi, int32_t plo, int32_t p
 
 // foot_count for up to two ranges a level and row: walks the elementary pieces of the cell from
 // left to right.
-WS_HD void foot_count_pieces(const FootHull &cur, const FootHull &prv, int32_t A, int32_t P, int32_t hmin,
+WS_FOOT void foot_count_pieces(const FootHull &cur, const FootHull &prv, int32_t A, int32_t P, int32_t hmin,
                              uint32_t mult, FootCounts &out) {
   int32_t c0, c1;
   foot_cell(A, P, hmin, c0, c1);
@@ -447,7 +435,7 @@ WS_HD void foot_count_pieces(const FootHull &cur, const FootHull &prv, int32_t A
 // covers the first level and the y set, the first one what only the z set reaches (empty when
 // its lines are counted on the wave, moved).  dmin / dmax: smallest and largest displacement.  Ranges of a
 // level's last row may reach into the cell after it.
-WS_HD void foot_targets(const FootGeo &g, int nl, int32_t dmin, int32_t dmax, bool z_alone, int32_t t[4]) {
+WS_FOOT void foot_targets(const FootGeo &g, int nl, int32_t dmin, int32_t dmax, bool z_alone, int32_t t[4]) {
   t[2] = g.rf[0] + dmin;
   t[3] = g.re[0] + dmax + 1;
   if (nl == 3 && g.lev[1].count > 0) {
@@ -468,7 +456,7 @@ WS_HD void foot_targets(const FootGeo &g, int nl, int32_t dmin, int32_t dmax, bo
 
 // Threads of blocks [0, n) of a candidate in launch order: `last` counts only those of the
 // last block row of each slab, `part` only those with fewer valid folded points than the fold.
-WS_HD_CALL int64_t foot_threads(const DCfg &c, int64_t n, bool last, bool part) {
+static __device__ __noinline__ int64_t foot_threads(const DCfg &c, int64_t n, bool last, bool part) {
   const uint32_t R = (uint32_t)n / (uint32_t)c.g[0];   // block ids stay below 2^31
   const int64_t gy = c.g[1], bz = R / (uint32_t)c.g[1];
   const int64_t bx = (uint32_t)n - R * (uint32_t)c.g[0], by = R - (uint32_t)bz * (uint32_t)c.g[1];
@@ -493,7 +481,7 @@ WS_HD_CALL int64_t foot_threads(const DCfg &c, int64_t n, bool last, bool part) 
 // Threads of the levels as sums of twelve such counts, term j of level j < 2 ? 0 : j < 6 ? 1 : 2
 // (wave, y set, z set): the wave's range; the y set's less its blocks in last block rows; the
 // z set's less what it shares with the y set.
-WS_HD int64_t foot_thread_term(const DCfg &c, int j, bool part) {
+WS_FOOT int64_t foot_thread_term(const DCfg &c, int j, bool part) {
   const bool has_y = c.y_hi > c.y_lo, has_z = c.z_hi > c.z_lo;
   const int64_t a = c.z_lo > c.y_lo ? c.z_lo : c.y_lo, b = c.z_hi < c.y_hi ? c.z_hi : c.y_hi;
   if ((j >= 2 && j < 6 && !has_y) || (j >= 6 && !has_z) || (j >= 8 && !(has_y && b > a))) return 0;
