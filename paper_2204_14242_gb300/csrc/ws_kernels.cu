@@ -2002,9 +2002,9 @@ __device__ __noinline__ void foot_field(const EnumArgs &a, FootSmem &m, const DF
   __syncwarp();
 }
 
-// The closed-form items of a pass: warps take fchunk consecutive ones at a time and keep the
-// geometry of a field group while they stay in it; before them each group's s_parts items for
-// what the walk does not count.
+// The closed-form items of a pass: warps take fchunk consecutive ones at a time (one, in plans of fewer
+// than some 34,000 mixed candidates) and make a field group's geometry anew unless the item before was of
+// the same one; before them each group's s_parts items for what the walk does not count.
 __device__ __forceinline__ void foot_items(const EnumArgs &a, FootSmem &m) {
   const uint32_t lane = threadIdx.x & 31u;
   int cur = -1;
@@ -2065,11 +2065,12 @@ __device__ __forceinline__ void foot_items(const EnumArgs &a, FootSmem &m) {
   }
 }
 
-// Row items first (CTAs), then the closed-form items (warps).  Bound by instruction fetch and the
-// latency of a warp's own chain: a unit runs a few thousand instructions once, so the code has to
-// stay in the SM's instruction cache (one copy of the walk, rare paths out of line), and two
-// CTAs an SM with 128 registers beat three or four that spill (0.23 against 0.29 and 0.35 ms,
-// 25-point sweep of 755).  Footprints of 755 25-point candidates at 640 x 512 x 512: 0.193 ms of
+// Row items first (CTAs), then the closed-form items (warps).  Bound by latency: with the four warps a
+// scheduler that 128 registers allow (3.3 to 3.6 active), issue slots are 31 to 43 % busy; per issue 2.5 warps
+// wait for the ALU result before, 1.3 to 2.8 for an instruction fetch (a unit runs a few thousand instructions
+// once) and 0.8 to 3.2 for memory (ncu: 755 25-point, 189 lattice Boltzmann, 400 mixed candidates).  So
+// there is one copy of the walk and rare paths are out of line, and two CTAs an SM with 128 registers
+// beat three or four that spill (0.23 against 0.29 and 0.35 ms, 25-point sweep of 755).  Footprints of 755 25-point candidates at 640 x 512 x 512: 0.193 ms of
 // red.or and 0.092 ms of counting 179 MB of bitmaps -> 0.230 and 0.018 ms; 755 lattice Boltzmann
 // candidates: 1.163 and 0.984 -> 0.252 and 0.002 ms (3.66 GB of bitmaps not read, fields that are
 // whole-line copies counted once); 4,000 mixed candidates: 2.66 and 1.32 -> 1.90 and 0.06 ms.
