@@ -168,7 +168,6 @@ struct ws_plan {
   // the bitmaps it fills (levels counted in closed form fill none)
   int64_t citems_accounted = 0;
   int32_t foot_chunk = 1;        // closed-form items a warp takes at once
-  int32_t foot_stat = 1;         // least items per group for what the closed-form walk does not count
   int64_t own_budget = 0;        // owner-table entries the descriptor estimate allows for
   size_t grab_bytes = 0, counters_bytes = 0;
   // uploaded arrays that the plan owns until it is destroyed (their copies are asynchronous)

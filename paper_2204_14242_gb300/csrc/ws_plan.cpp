@@ -286,7 +286,7 @@ struct Compiled {
   std::pmr::vector<uint64_t> fkey;  // (field index, folding): equal keys have equal access lists
   std::pmr::vector<int64_t> need_words;  // bitmap words per field
   size_t dsc_bytes = 0;             // descriptor bytes of its fields, lists and groups
-  size_t dsp_bytes = 0;             // bytes of their displacements
+  size_t dsp_bytes = 0;             // bytes of their displacements and work counters (descriptor_extra)
   size_t need_sum = 0, need_max = 0;  // bitmap bytes of all its fields / of its largest
   size_t items_est = 0;             // bound on its work items (owner table entries)
   int64_t n_acc_own = 0, n_iv_own = 0;  // list entries of its fields that no other candidate shares
@@ -1457,11 +1457,12 @@ static constexpr int64_t kFootUnitMin = 1000, kFootUnitSmall = 10000, kFootUnitM
                          kFootPerWarp = 3;
 
 // What the closed-form walk does not count of a group (foot_stats) goes over the row slots of its wave, some
-// 0.5 us for 32 of them in one warp.  Up to eight items a group where there are few groups, and as many as
-// share the plan's slots out four to a resident warp, of at least kStatSlotsMin (the plain form: just that)
-// and at most kStatSlotsMax slots: with eight items whatever the wave, one 7-point candidate with a wave of 400,000
-// blocks of 4 x 8 x 4 took 228 us a step, now 93; 4,000 mixed candidates 2.27 and 2.23 ms (GB300).
-static constexpr int64_t kStatSlotsMin = 256, kStatSlotsMax = 8192;
+// 0.5 us for 32 of them in one warp, in items of kStatSlotsMin to kStatSlots slots (the fewest where all the
+// plan's waves have few), more where that makes over four items a resident warp, at most kStatSlotsMax.  One
+// 7-point candidate with a wave of 400,000 blocks of 4 x 8 x 4 takes 92 us a step, in eight items 228; 755
+// lattice Boltzmann candidates 318 us, in items of 128 slots 338; twelve served requests 55.6 us of rows_kernel
+// on average, in items of 256 slots 57.4 (GB300).
+static constexpr int64_t kStatSlotsMin = 128, kStatSlots = 256, kStatSlotsMax = 8192;
 
 // Numbers work items and cuts passes for the current tuning.
 // Runs fn(lo, hi) over [0, n) in chunks on the host pool (defined with the pool below).
@@ -1542,7 +1543,7 @@ void ws_plan::layout() {
   // closed-form items: a field's units are shared out among parts of foot_unit estimated warp
   // instructions (kFootPerWarp and its neighbours; two CTAs of eight warps are resident per SM),
   // without exceeding the owner-table entries the descriptor estimate allowed for
-  int64_t foot_unit = kFootUnitMin, stat_slots = kStatSlotsMax;
+  int64_t foot_unit = kFootUnitMin, stat_slots = kStatSlotsMin;
   {
     const int64_t warps = 16 * (int64_t)(ctx ? ctx->sm_count : 152);
     int64_t cost = 0, fields = 0;
@@ -1559,15 +1560,12 @@ void ws_plan::layout() {
     if (own_budget > 0) foot_unit = std::max(foot_unit, cost / std::max<int64_t>(1, own_budget / 2));
     foot_chunk = (int32_t)std::max<int64_t>(1, std::min<int64_t>(8, fields / (64 * warps)));
     if (plain_layout) foot_chunk = 1;
-    int foot_groups = 0;
     int64_t wave_slots = 0;
-    for (int g = 0; g < ng; ++g) {
-      foot_groups += hgrp[(size_t)g].foot != 0;
+    for (int g = 0; g < ng; ++g)
       if (hgrp[(size_t)g].foot & 1) wave_slots += grp_wave_slots[(size_t)g];
-    }
-    stat_slots = plain_layout ? kStatSlotsMin : std::max(kStatSlotsMin, std::min(kStatSlotsMax, wave_slots / (4 * warps)));
-    const int64_t share = 4 * warps / std::max<int64_t>(1, plain_layout ? 1 : foot_groups);
-    foot_stat = (int32_t)std::max<int64_t>(1, std::min<int64_t>(8, share));
+    if (!plain_layout)
+      stat_slots = std::max({stat_slots, std::min(4 * wave_slots / warps, kStatSlots),
+                             std::min(wave_slots / (4 * warps), kStatSlotsMax)});
   }
   // passes (a group starts a new one when its words would overflow the capacity), each
   // group's first scratch word in its pass, and the enumeration and row-walk items: the
@@ -1618,7 +1616,7 @@ void ws_plan::layout() {
       G.f_parts = G.foot ? (uint8_t)std::max<int64_t>(1, std::min<int64_t>(kFootParts, grp_foot_cost[(size_t)g] / foot_unit)) : 0;
       fitems += (int64_t)__builtin_popcount(G.foot_fields) * G.f_parts;
       G.sitem_begin = (int32_t)sitems;
-      G.s_parts = G.foot & 1 ? (int32_t)std::max<int64_t>(foot_stat, ceil_div(grp_wave_slots[(size_t)g], stat_slots)) : 0;
+      G.s_parts = G.foot & 1 ? (int32_t)ceil_div(grp_wave_slots[(size_t)g], stat_slots) : 0;
       sitems += G.s_parts;
       walk_work += row_slots(g) * (G.n_iv + G.n_stores);
       if (G.foot) foot_work += grp_foot_cost[(size_t)g] * __builtin_popcount(G.foot_fields);
@@ -1819,15 +1817,14 @@ int ws_plan::bank_shift() const {
 }
 
 // CTAs of rows_kernel (of its instance without closed-form items where there are none): one per
-// row-walk item, one per eight warps' closed-form items.
+// row-walk item, or per closed-form item (a small call's are spread over the SMs).
 int ws_plan::grid_rows(int64_t items, int64_t fitems, int64_t sitems) const {
   int occ = 1;
   rows_occupancy(iv_cap, fitems > 0, &occ);
   if (tune.ctas_per_sm > 0) occ = std::min(occ, tune.ctas_per_sm);
   occ = std::max(occ, 1);
   int64_t g = (int64_t)ctx->sm_count * occ;
-  const int64_t witems = std::max(fitems * (1 + foot_stat), fitems + sitems);
-  items = std::max(items, ceil_div(witems, (int64_t)foot_chunk * (kRowsThreads / 32)));
+  items = std::max(items, ceil_div(fitems + sitems, (int64_t)foot_chunk));
   g = std::min<int64_t>(g, std::max<int64_t>(items, 1));
   return (int)g;
 }
@@ -2312,6 +2309,9 @@ static void parallel_chunks(int64_t n, int64_t chunk, const std::function<void(i
   });
 }
 
+// Four work-stealing counters per pass (enumeration, row walk, counting, closed form).
+constexpr size_t kGrabBytes = 4 * sizeof(unsigned long long);
+
 static void compile_all(const ws_config *cfgs, int n_cfg, const ws_field *fld, int n_fld, const ws_access *acc,
                         int n_acc, const ws_hw &hw, int64_t chunk_warps, CompileArena &ca, std::vector<int> &status) {
   ca.comp.assign(n_cfg, nullptr);
@@ -2354,7 +2354,7 @@ static void compile_all(const ws_config *cfgs, int n_cfg, const ws_field *fld, i
         const size_t cr = 256;   // the smallest row-walk item
         for (size_t k = 0; k < cc.f.size(); ++k) {
           const int64_t nacc = cc.acc_off[k + 1] - cc.acc_off[k], niv = cc.iv_off[k + 1] - cc.iv_off[k];
-          cc.dsp_bytes += (size_t)(cc.f[k].n_dsp_l + cc.f[k].n_dsp_s) * sizeof(DDsp);   // (descriptor_extra)
+          cc.dsp_bytes += (size_t)(cc.f[k].n_dsp_l + cc.f[k].n_dsp_s) * sizeof(DDsp) + kGrabBytes;
           cc.dsc_bytes += sizeof(DField) + sizeof(DGroup) + (size_t)nacc * sizeof(DAcc) +
                           (size_t)cc.f[k].n_iv * sizeof(DIv);
           cc.need_sum += (size_t)cc.need_words[k] * 4;
@@ -2397,9 +2397,6 @@ int ws::plan_requirements(const ws_config *cfgs, int n_cfg, const ws_field *fld,
   *scratch_bytes = scr;
   return WS_OK;
 }
-
-// Four work-stealing counters per pass (enumeration, row walk, counting, closed form).
-constexpr size_t kGrabBytes = 4 * sizeof(unsigned long long);
 
 // Host half of plan creation: compiles the candidates, deduplicates their access lists,
 // builds field groups and cuts passes.  avail_fn(descriptor bytes, bitmap bytes of all
@@ -2608,11 +2605,9 @@ constexpr size_t kDescHeadroom = (size_t)8 << 20;
 // closed form's displacements, which grow with the accesses (1,500 fields of 961 loads in rows of
 // their own have 23 MB).  Only what the headroom cannot hold is added, so that a batch that fits a
 // given arena without them still does.
-static size_t descriptor_extra(const CompileArena &ca, const std::vector<int> &status) {
+// bytes: of all candidates, shared lists as often as they are shared.
+static size_t descriptor_extra(const CompileArena &ca, const std::vector<int> &status, size_t bytes) {
   const size_t room = kDescHeadroom - ((size_t)256 << 10);   // (the rest: granularity of the buffers)
-  size_t bytes = 0;
-  for (size_t i = 0; i < status.size(); ++i)
-    if (status[i] == WS_OK) bytes += ca.comp[i]->dsp_bytes + kGrabBytes * ca.comp[i]->f.size();
   if (bytes <= room) return 0;
   std::unordered_set<uint64_t> seen;   // (seldom) the shared lists once
   for (size_t i = 0; i < status.size(); ++i) {
@@ -2639,10 +2634,11 @@ static void build_host(Plan *p, const ws_config *cfgs, int n_cfg, const ws_field
   const std::vector<Compiled *> &comp = ca.comp;
   // scratch capacity: what the arena can give after the descriptors (a field, its access
   // and interval lists, at most one field group each)
-  size_t dsc = 64 * 1024, total_need = 0, max_field = 0;
+  size_t dsc = 64 * 1024, total_need = 0, max_field = 0, extra = 0;
   for (int i = 0; i < n_cfg; ++i) {
     if (status[i] != WS_OK) continue;
     dsc += comp[i]->dsc_bytes;
+    extra += comp[i]->dsp_bytes;
     total_need += comp[i]->need_sum;
     max_field = std::max(max_field, comp[i]->need_max);
   }
@@ -2659,7 +2655,7 @@ static void build_host(Plan *p, const ws_config *cfgs, int n_cfg, const ws_field
     dsc += 4 * 3 * items;
     p->own_budget = (int64_t)(3 * items);
   }
-  dsc += descriptor_extra(ca, status);
+  dsc += descriptor_extra(ca, status, extra);
   const size_t avail = avail_fn(dsc, total_need);
   size_t scratch = std::min(total_need, avail);
   scratch = std::max<size_t>(scratch, 16);

@@ -1,6 +1,6 @@
 """Waves of many row slots: what the closed form does not count is shared out by their number.
 
-A slot is one thread row of one block row; in a batch of fewer than 2.5 million of them an item takes
+A slot is one thread row of one block row; in a batch of fewer than 2.4 million of them an item takes
 at most 256.
 """
 import pytest
