@@ -212,8 +212,7 @@ namespace ws {
 using Plan = ::ws_plan;
 
 int plan_requirements(const ws_config *cfgs, int n_cfg, const ws_field *fld, int n_fld, const ws_access *acc,
-                      int n_acc, const ws_hw *hw, size_t *desc_bytes, size_t *scratch_bytes,
-                      size_t *max_field_bytes);
+                      int n_acc, const ws_hw *hw, size_t *scratch_bytes, size_t *max_field_bytes);
 // ext_scratch value of plan_create_impl: use (and grow) the context's kept one-shot scratch;
 // the caller holds ctx->oneshot_mu.
 constexpr int64_t kCtxScratch = -2;

@@ -334,9 +334,9 @@ extern "C" int ws_server_submit(ws_server *s, const ws_request *req, uint64_t *r
   r->cfgs.assign(req->cfgs, req->cfgs + req->n_cfg);
   r->fld.assign(req->fld, req->fld + req->n_fld);
   r->acc.assign(req->acc, req->acc + req->n_acc);
-  size_t dsc = 0, scr = 0, mf = 0;
+  size_t scr = 0, mf = 0;
   ws::plan_requirements(r->cfgs.data(), req->n_cfg, r->fld.data(), req->n_fld, r->acc.data(), req->n_acc, &s->hw,
-                        &dsc, &scr, &mf);
+                        &scr, &mf);
   r->scratch_bytes = scr;
   r->max_field_bytes = mf;
   std::lock_guard<std::mutex> g(s->mu);
