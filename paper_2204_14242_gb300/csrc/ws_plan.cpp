@@ -327,6 +327,7 @@ struct RunRow {
 struct FieldFold {
   int status = WS_OK;
   std::vector<DAcc> da;
+  bool runs = false;        // the merged load runs are made
   std::vector<DIv> iv;      // merged load runs, then the displacements of the closed form
   std::vector<RunRow> rr;   // the runs' grid rows
   // for the row walk (cover_runs): the runs without a covering run, those covered from another z
@@ -445,9 +446,12 @@ static void field_displacements(const ws_field &F, FieldFold &out) {
   }
 }
 
-// sizes: only what the bitmaps' sizes and the candidate's status depend on (the accesses' number and range).
+// What a field compiles to: what the bitmaps' sizes and the candidate's status depend on (the accesses'
+// number and range); all but the merged load runs, which fields counted in closed form do not read; all.
+enum Lists { kSizes, kClosed, kRuns };
+
 static void compile_field_fold(const ws_field &F, const ws_access *acc, int n_acc, int fold_axis, int fold,
-                               FieldFold &out, bool sizes = false) {
+                               FieldFold &out, Lists lists) {
   out.status = WS_OK;
   if (F.elem_bytes < 1 || F.elem_bytes > 64 || F.n_access < 1 || F.access_off < 0 ||
       F.access_off + F.n_access > n_acc) {
@@ -513,11 +517,16 @@ static void compile_field_fold(const ws_field &F, const ws_access *acc, int n_ac
     }
   out.n_load = (int32_t)lk.size();
   out.n_store = (int32_t)sk.size();
-  if (sizes) return;
+  if (lists == kSizes) return;
+  out.rr.clear();
+  out.iv.clear();
+  out.iv_cov.clear();
+  out.covered = false;
+  out.runs = lists == kRuns;
   // merged load intervals: sorted load offsets cut wherever two neighbours are more than
   // 32 B apart (a chain of byte addresses with steps of at most 32 B touches every
   // sector between its ends); for each, the grid row of its offsets
-  {
+  if (out.runs) {
     struct Ld {
       int64_t b, o[4];   // byte offset; dx dy dz dc
     };
@@ -529,10 +538,6 @@ static void compile_field_fold(const ws_field &F, const ws_access *acc, int n_ac
     }
     std::sort(b.begin(), b.end(), [](const Ld &p, const Ld &q) { return p.b < q.b; });
     std::vector<RunRow> &rr = out.rr;
-    rr.clear();
-    out.iv.clear();
-    out.iv_cov.clear();
-    out.covered = false;
     for (size_t i = 0; i < b.size();) {
       size_t j = i;
       while (j + 1 < b.size() && b[j + 1].b - b[j].b <= 32) ++j;
@@ -566,8 +571,7 @@ static void compile_field_fold(const ws_field &F, const ws_access *acc, int n_ac
   }
 }
 
-// Finds the runs' covering runs.  Only the row walk reads them, so candidates counted in closed form
-// throughout leave them out (finding them is a third of the time a field takes to compile).
+// Finds the runs' covering runs, which only the row walk reads.
 static void cover_runs(int fold_axis, int fold, FieldFold &out) {
   if (out.covered) return;
   out.covered = true;
@@ -868,13 +872,16 @@ static uint64_t fold_key(const ws_config &c, int fi) {
 }
 static const uint64_t kNoShare = ~(uint64_t)0;   // a list that no other descriptor shares
 static const uint64_t kCoveredKey = (uint64_t)1 << 63;   // the list with the covering runs
+static const uint64_t kRunsKey = (uint64_t)1 << 62;      // the list with the merged load runs
 
 // Returns WS_OK or a per-candidate error status.  `cache` (may be null) memoizes the
-// per-(field, folding) part across candidates that share fields.  sizes: only the status and
-// out.need_words are made.
+// per-(field, folding) part across candidates that share fields.  lists: what is made of the
+// fields' lists; with kSizes only the status and out.need_words, with kClosed the merged load runs
+// of candidates that some walk reads them for.
 static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, const ws_access *acc, int n_acc,
                           const ws_hw &hw, Compiled &out, FieldCache *cache = nullptr,
-                          const uint8_t *field_refs = nullptr, bool sizes = false) {
+                          const uint8_t *field_refs = nullptr, Lists lists = kClosed) {
+  const bool sizes = lists == kSizes;
   DCfg &d = out.d;
   memset(&d, 0, sizeof(d));
   for (int k = 0; k < 3; ++k) {
@@ -1108,10 +1115,17 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     }
     return run_min[lv];
   };
-  // A candidate whose levels are all counted in closed form (or by the address walk) needs no
-  // covering runs; a field that the row walk takes turns them on and starts the candidate again.
-  const int kNeedsCovers = INT_MIN;
-  bool covers = false;
+  // A candidate whose levels are all counted in closed form (or by the address walk) needs no merged
+  // runs; a field that a walk reads them for turns them on, and their covering runs where it is the row
+  // walk, and starts the candidate again.
+  const int kAgain = INT_MIN;
+  bool runs = lists == kRuns, covers = false;
+  if (lists == kClosed && c.address_mode == WS_ADDR_LINEAR) {
+    // at once where the first field's rows descend, or its planes are no whole number of rows apart
+    const ws_field &F = fld[c.field_off];
+    const bool planes = F.stride[1] > 0 && F.stride[2] % F.stride[1] == 0;
+    runs = covers = F.stride[1] <= 0 || F.stride[0] < 0 || (!planes && pb_hi[1][2] > pb_lo[1][2]);
+  }
   auto emit = [&](const ws_field &F, const FieldFold *ff, int mask, uint64_t key, bool first) -> int {
     const bool cover = covers && ff->covered;
     DField df;
@@ -1193,8 +1207,8 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     // 32-bit offsets, so the wave bitmap must span less than 2^31 bytes
     df.iv = (!df.wide && df.words[1] < ((int64_t)1 << 21) && std::llabs(F.stride[0]) * F.elem_bytes <= 32) ? 1 : 0;
     df.iv_begin = 0;
-    df.n_iv = ff->n_iv;
-    df.n_iv_unc = cover ? ff->n_iv_unc : ff->n_iv;
+    df.n_iv = runs ? ff->n_iv : 0;
+    df.n_iv_unc = cover ? ff->n_iv_unc : df.n_iv;
     if (cover) {
       df.n_iv_zc = ff->n_iv_zc;
       df.cov_dy = ff->cov_dy;
@@ -1241,23 +1255,29 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     const bool dsp = df.closed != 0 || key != kNoShare;
     if (!dsp) df.n_dsp_l = df.n_dsp_s = 0;
     out.f.push_back(df);
-    out.iv.insert(out.iv.end(), iv.begin(), dsp ? iv.end() : iv.begin() + ff->n_iv);
+    out.iv.insert(out.iv.end(), iv.begin() + (runs ? 0 : ff->n_iv), dsp ? iv.end() : iv.begin() + ff->n_iv);
     out.acc_off.push_back((int32_t)out.acc.size());
     out.iv_off.push_back((int32_t)out.iv.size());
-    out.fkey.push_back(key != kNoShare && cover ? key | kCoveredKey : key);
+    out.fkey.push_back(key == kNoShare ? key : key | (runs ? kRunsKey : 0) | (cover ? kCoveredKey : 0));
     const int all = (mask & 1 ? 2 : 0) | (mask & 2 ? 1 : 0);
-    return !covers && out.rows_geom_ok && df.iv && df.rows_ok && df.closed != all ? kNeedsCovers : WS_OK;
+    const bool rows = out.rows_geom_ok && df.rows_ok;
+    if (lists == kRuns || !df.iv || (rows && df.closed == all)) return WS_OK;
+    const bool again = !runs || (rows && !covers);
+    runs = true;
+    covers = covers || rows;
+    return again ? kAgain : WS_OK;
   };
   // the folded lists of field fi: from the cache when other candidates use the field too,
   // else compiled into `local` (then *own = true: the list is this candidate's alone);
   // tl_fold is this thread's reusable one
   static thread_local FieldFold tl_fold;
   int local_field = -1;   // the field it holds
+  auto made = [&]() { return sizes ? kSizes : runs ? kRuns : kClosed; };
   auto fold_of = [&](int fi, FieldFold &local, bool *own) -> FieldFold * {
     const ws_field &F = fld[c.field_off + fi];
     *own = !cache || (field_refs && field_refs[c.field_off + fi] < 2);
     if (*own) {
-      if (local_field != fi) compile_field_fold(F, acc, n_acc, c.fold_axis, c.fold, local, sizes);
+      if (local_field != fi || (runs && !local.runs)) compile_field_fold(F, acc, n_acc, c.fold_axis, c.fold, local, made());
       local_field = fi;
       if (covers && local.status == WS_OK) cover_runs(c.fold_axis, c.fold, local);
       return &local;
@@ -1265,7 +1285,9 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     auto it = cache->find(fold_key(c, fi));
     if (it == cache->end()) {
       it = cache->emplace(fold_key(c, fi), FieldFold()).first;
-      compile_field_fold(F, acc, n_acc, c.fold_axis, c.fold, it->second, sizes);
+      compile_field_fold(F, acc, n_acc, c.fold_axis, c.fold, it->second, made());
+    } else if (runs && it->second.status == WS_OK && !it->second.runs) {
+      compile_field_fold(F, acc, n_acc, c.fold_axis, c.fold, it->second, kRuns);
     }
     if (covers && it->second.status == WS_OK) cover_runs(c.fold_axis, c.fold, it->second);
     return &it->second;
@@ -1334,7 +1356,7 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
         V.stride[1] = (int64_t)(RS / F.elem_bytes);
         V.stride[2] = (int64_t)(PS / F.elem_bytes);
         V.align_bytes = (int64_t)(xbias[fi] - RS * ymin - PS * zmin);
-        compile_field_fold(V, acc, n_acc, c.fold_axis, c.fold, tl_fold, sizes);
+        compile_field_fold(V, acc, n_acc, c.fold_axis, c.fold, tl_fold, made());
         local_field = -1;
         if (tl_fold.status != WS_OK) return tl_fold.status;
         if (covers) cover_runs(c.fold_axis, c.fold, tl_fold);
@@ -1344,9 +1366,8 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     }
     return WS_OK;
   };
-  int rc = emit_all();
-  if (rc == kNeedsCovers) {
-    covers = true;
+  int rc;
+  while ((rc = emit_all()) == kAgain) {   // (twice at most)
     out.f.clear();
     out.acc.clear();
     out.iv.clear();
@@ -1354,7 +1375,6 @@ static int compile_config(const ws_config &c, const ws_field *fld, int n_fld, co
     out.iv_off.resize(1);
     out.fkey.clear();
     out.need_words.clear();
-    rc = emit_all();
   }
   if (rc != WS_OK) return rc;
   d.n_field = c.n_field;
@@ -2316,7 +2336,9 @@ static void parallel_chunks(int64_t n, int64_t chunk, const std::function<void(i
 constexpr size_t kGrabBytes = 4 * sizeof(unsigned long long);
 
 static void compile_all(const ws_config *cfgs, int n_cfg, const ws_field *fld, int n_fld, const ws_access *acc,
-                        int n_acc, const ws_hw &hw, int64_t chunk_warps, CompileArena &ca, std::vector<int> &status) {
+                        int n_acc, const ws_hw &hw, const ws_tuning &tune, CompileArena &ca, std::vector<int> &status) {
+  const int64_t chunk_warps = std::max(1, tune.chunk_warps);
+  const Lists lists = tune.walk == WS_WALK_INTERVAL ? kClosed : kRuns;   // (the other walks take every field)
   ca.comp.assign(n_cfg, nullptr);
   status.assign(n_cfg, WS_OK);
   // chunks of consecutive candidates handed out dynamically; each thread keeps its fold
@@ -2351,7 +2373,7 @@ static void compile_all(const ws_config *cfgs, int n_cfg, const ws_field *fld, i
       for (int i = c * chunk; i < std::min(n_cfg, (c + 1) * chunk); ++i) {
         Compiled &cc = *new (r->allocate(sizeof(Compiled), alignof(Compiled))) Compiled(r);
         ca.comp[(size_t)i] = &cc;
-        status[i] = compile_config(cfgs[i], fld, n_fld, acc, n_acc, hw, cc, &cache, refs.data());
+        status[i] = compile_config(cfgs[i], fld, n_fld, acc, n_acc, hw, cc, &cache, refs.data(), lists);
         if (status[i] != WS_OK) continue;
         const DCfg &d = cc.d;
         const size_t cr = 256;   // the smallest row-walk item
@@ -2387,7 +2409,7 @@ int ws::plan_requirements(const ws_config *cfgs, int n_cfg, const ws_field *fld,
   FieldCache cache;
   for (int i = 0; i < n_cfg; ++i) {
     Compiled cc;
-    if (compile_config(cfgs[i], fld, n_fld, acc, n_acc, *hw, cc, &cache, nullptr, true) != WS_OK) continue;
+    if (compile_config(cfgs[i], fld, n_fld, acc, n_acc, *hw, cc, &cache, nullptr, kSizes) != WS_OK) continue;
     for (int64_t words : cc.need_words) {
       scr += (size_t)words * 4;
       mf = std::max(mf, (size_t)words * 4);
@@ -2630,7 +2652,7 @@ static void build_host(Plan *p, const ws_config *cfgs, int n_cfg, const ws_field
   p->cfg_cf_begin.assign(n_cfg + 1, 0);
   CompileArena ca;
   std::vector<int> status;
-  compile_all(cfgs, n_cfg, fld, n_fld, acc, n_acc, *hw, std::max(1, p->tune.chunk_warps), ca, status);
+  compile_all(cfgs, n_cfg, fld, n_fld, acc, n_acc, *hw, p->tune, ca, status);
   const std::vector<Compiled *> &comp = ca.comp;
   // scratch capacity: what the arena can give after the descriptors (a field, its access
   // and interval lists, at most one field group each)
