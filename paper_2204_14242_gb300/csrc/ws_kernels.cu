@@ -2066,14 +2066,14 @@ __device__ __forceinline__ void foot_items(const EnumArgs &a, FootSmem &m) {
 }
 
 // Row items first (CTAs), then the closed-form items (warps).  Bound by latency: with the four warps a
-// scheduler that 128 registers allow (3.3 to 3.6 active), issue slots are 31 to 43 % busy; per issue 2.5 warps
-// wait for the ALU result before, 1.3 to 2.8 for an instruction fetch (a unit runs a few thousand instructions
-// once) and 0.8 to 3.2 for memory (ncu: 755 25-point, 189 lattice Boltzmann, 400 mixed candidates).  So
+// scheduler that 128 registers allow (3.3 to 3.6 active), issue slots are 32 to 42 % busy; per issue 2.5 warps
+// wait for the ALU result before, 1.3 to 3.3 for an instruction fetch (a unit runs a few thousand instructions
+// once) and 0.6 to 2.2 for memory (ncu: 755 25-point, 189 lattice Boltzmann, 400 mixed candidates).  So
 // there is one copy of the walk and rare paths are out of line, and two CTAs an SM with 128 registers
 // beat three or four that spill (0.23 against 0.29 and 0.35 ms, 25-point sweep of 755).  Footprints of 755 25-point candidates at 640 x 512 x 512: 0.193 ms of
-// red.or and 0.092 ms of counting 179 MB of bitmaps -> 0.230 and 0.018 ms; 755 lattice Boltzmann
-// candidates: 1.163 and 0.984 -> 0.252 and 0.002 ms (3.66 GB of bitmaps not read, fields that are
-// whole-line copies counted once); 4,000 mixed candidates: 2.66 and 1.32 -> 1.90 and 0.06 ms.
+// red.or and 0.092 ms of counting 179 MB of bitmaps -> 0.221 and 0.023 ms; 755 lattice Boltzmann
+// candidates: 1.163 and 0.984 -> 0.229 and 0.002 ms (3.66 GB of bitmaps not read, fields that are
+// whole-line copies counted once); 4,000 mixed candidates: 2.66 and 1.32 -> 1.89 and 0.08 ms.
 // Without closed-form items the row walk has an instance of its own, 64 registers and four CTAs an
 // SM: 755 25-point candidates with descending rows 0.287 -> 0.196 ms, 755 lattice Boltzmann ones whose
 // planes are no whole number of rows apart 1.84 -> 1.46 ms.

@@ -1484,8 +1484,9 @@ static constexpr int64_t kFootUnitMin = 1000, kFootUnitSmall = 10000, kFootUnitM
 // plan's waves have few), more where that makes over four items a resident warp, at most kStatSlotsMax.  One
 // 7-point candidate with a wave of 400,000 blocks of 4 x 8 x 4 takes 92 us a step, in eight items 228; 755
 // lattice Boltzmann candidates 318 us, in items of 128 slots 338; twelve served requests 55.6 us of rows_kernel
-// on average, in items of 256 slots 57.4 (GB300).
-static constexpr int64_t kStatSlotsMin = 128, kStatSlots = 256, kStatSlotsMax = 8192;
+// on average, in items of 256 slots 57.4.  The plain form, one candidate a launch, takes kStatSlotsPlain (151
+// lattice Boltzmann candidates 9.54 ms, with 128 slots 9.64, with 1024 11.7; GB300).
+static constexpr int64_t kStatSlotsMin = 128, kStatSlots = 256, kStatSlotsMax = 8192, kStatSlotsPlain = 64;
 
 // Numbers work items and cuts passes for the current tuning.
 // Runs fn(lo, hi) over [0, n) in chunks on the host pool (defined with the pool below).
@@ -1586,7 +1587,8 @@ void ws_plan::layout() {
     int64_t wave_slots = 0;
     for (int g = 0; g < ng; ++g)
       if (hgrp[(size_t)g].foot & 1) wave_slots += grp_wave_slots[(size_t)g];
-    if (!plain_layout)
+    if (plain_layout) stat_slots = kStatSlotsPlain;
+    else
       stat_slots = std::max({stat_slots, std::min(4 * wave_slots / warps, kStatSlots),
                              std::min(wave_slots / (4 * warps), kStatSlotsMax)});
   }
